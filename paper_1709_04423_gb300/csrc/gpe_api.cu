@@ -324,6 +324,13 @@ int upload_coefs_t(gp_handle* h) {
                     tabs.data() + (size_t)si * 512, n, kSegs[si], 1, tau, h->cdepth[mode][d][si], pts);
         h->cpts[mode][d][si] = carry_pts_class(pts);
       }
+      if (h->dim == 1) {
+        // the points after which a product of the coefficients is below the threshold
+        double amax = 0.0;
+        for (int k = 1; k <= n - 2; ++k) amax = std::max({amax, std::abs(af[k]), std::abs(ab[k])});
+        const double r = amax < 1.0 ? std::ceil(std::log(tau) / std::log(std::max(amax, 1e-300))) : (double)n;
+        h->line_reach[mode] = (long)std::min<double>(std::max(r, 1.0), (double)n);
+      }
       int rc = upload_c2<T>(h, h->coef[mode][d], all);
       if (rc) return rc;
       if ((rc = upload_c2<T>(h, h->ctab[mode][d], tabs))) return rc;
@@ -480,6 +487,12 @@ int upload_coefs(gp_handle* h) {
 
 // Step launchers of the handle's state precision.
 int run_steps_any(gp_handle* h, bool imag, long nsteps) {
+  if (h->dim == 1 && nsteps > 0) {
+    const int rc = h->prec == GP_DF64  ? run_line_df(h, imag, nsteps)
+                   : h->prec == GP_F64 ? run_line_f64(h, imag, nsteps)
+                                       : run_line_f32(h, imag, nsteps);
+    if (rc != GP_ERR_STATE) return rc;
+  }
   if (h->prec == GP_DF64) return run_steps_df(h, imag, nsteps);
   return h->prec == GP_F64 ? run_steps_f64(h, imag, nsteps) : run_steps_f32(h, imag, nsteps);
 }

@@ -107,6 +107,8 @@ struct gp_handle {
   // per mode, axis and segment length: the segment carries' reach (Sweep2Args cdepth, cpts)
   int cdepth[gpe::NUM_MODES][3][gpe::kNumSegs] = {};
   int cpts[gpe::NUM_MODES][3][gpe::kNumSegs] = {};
+  // 1d grids: points over which a carry falls below the precision's threshold
+  long line_reach[gpe::NUM_MODES] = {0};
   // circular / axial traps (geom 2): per mode, the rho axis' backward
   // coefficients, forward right-hand-side factors and stencil factors
   // (vab, vbf, vh of Sweep2Args; 3 n[0] complex values)
@@ -252,6 +254,10 @@ void launch_df_to_c128(void* dst, const void* src, long n, cudaStream_t s);
 void materialize_complex(gp_handle* h);
 int real_from_complex(gp_handle* h);
 void tf_from_c128(gp_handle* h, void* dst, const void* src, long n);  // exact triple-float split
+// every step of a 1d grid in one launch (gpe_line.cuh); GP_ERR_STATE: the line is too long for it
+int run_line_f32(gp_handle* h, bool imag, long nsteps);
+int run_line_f64(gp_handle* h, bool imag, long nsteps);
+int run_line_df(gp_handle* h, bool imag, long nsteps);
 int run_steps_f32(gp_handle* h, bool imag, long nsteps);
 int run_steps_f64(gp_handle* h, bool imag, long nsteps);
 int time_steps_f32(gp_handle* h, bool imag, long nsteps, double* ms_out);

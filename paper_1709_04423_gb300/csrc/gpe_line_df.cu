@@ -1,0 +1,8 @@
+// gpe_line_df.cu -- instantiates the one-launch stepping of 1d grids for the df64 state.
+#include "gpe_line.cuh"
+
+namespace gpe {
+
+int run_line_df(gp_handle* h, bool imag, long nsteps) { return run_line_t<df64>(h, imag, nsteps); }
+
+}  // namespace gpe

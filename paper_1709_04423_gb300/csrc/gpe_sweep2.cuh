@@ -199,6 +199,70 @@ __device__ __forceinline__ c2_t<T> phase_N(c2_t<T> p, c2_t<T> F, T dtg) {
   }
 }
 
+// FP64 sub-step N from the whole angle th = dt (V + g |p|^2): p <- exp(-i th) p
+// as rot_apply does, p + ((cos th - 1) p + sin th (p.y, -p.x)), or p <- p +
+// (exp(-th) - 1) p.  The coefficients are Taylor series -- for |th| < 1/32 sin to
+// th^7, cos - 1 to th^8, exp - 1 to th^8, for |th| < 1/4 to th^11, th^12, th^12
+// (first omitted terms below 1e-17 of the coefficient) -- else the library
+// functions.  A rounded factor next to 1 (F above) repeats its own rounding at a
+// point step after step; here only the small coefficient is rounded, and the
+// sum's rounding is unbiased.  19 FP64 operations per point against 24 in real
+// time, 13 against 15 in imaginary time.
+template <bool IMAG>
+__device__ __forceinline__ double2 phase_theta(double2 p, double th) {
+  if (IMAG) {
+    const double m = -th;
+    double t;
+    if (fabs(th) < 0.03125) {
+      t = 1.0 / 40320;
+      t = fma(m, t, 1.0 / 5040);
+      t = fma(m, t, 1.0 / 720);
+    } else if (fabs(th) < 0.25) {
+      t = 1.0 / 479001600;
+      t = fma(m, t, 1.0 / 39916800);
+      t = fma(m, t, 1.0 / 3628800);
+      t = fma(m, t, 1.0 / 362880);
+      t = fma(m, t, 1.0 / 40320);
+      t = fma(m, t, 1.0 / 5040);
+      t = fma(m, t, 1.0 / 720);
+    } else {
+      const double f = exp(m);
+      return make_double2(f * p.x, f * p.y);
+    }
+    t = fma(m, t, 1.0 / 120);
+    t = fma(m, t, 1.0 / 24);
+    t = fma(m, t, 1.0 / 6);
+    t = fma(m, t, 1.0 / 2);
+    t = fma(m, t, 1.0);
+    t = m * t;
+    return make_double2(fma(t, p.x, p.x), fma(t, p.y, p.y));
+  } else {
+    const double t2 = th * th;
+    double s, c;
+    if (fabs(th) < 0.03125) {
+      s = -1.0 / 5040;
+      c = 1.0 / 40320;
+      c = fma(t2, c, -1.0 / 720);
+    } else if (fabs(th) < 0.25) {
+      s = -1.0 / 39916800;
+      s = fma(t2, s, 1.0 / 362880);
+      s = fma(t2, s, -1.0 / 5040);
+      c = 1.0 / 479001600;
+      c = fma(t2, c, -1.0 / 3628800);
+      c = fma(t2, c, 1.0 / 40320);
+      c = fma(t2, c, -1.0 / 720);
+    } else {
+      return rot_neg<double>(p, th);
+    }
+    s = fma(t2, s, 1.0 / 120);
+    s = fma(t2, s, -1.0 / 6);
+    s = th * fma(t2, s, 1.0);
+    c = fma(t2, c, 1.0 / 24);
+    c = t2 * fma(t2, c, -1.0 / 2);
+    return rot_apply<double>(p, s, c);
+  }
+}
+
 // FP32 state: p <- exp(-i th) p or exp(-th) p with th = dt (V + g |p|^2)
 // formed per point (library sincos / exp of the state precision).  Real time
 // rotates with rot_neg, whose rounded rotation keeps |p| unbiased.
