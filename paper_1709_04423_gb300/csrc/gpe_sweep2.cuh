@@ -65,13 +65,13 @@ struct Sweep2Args {
   const c2_t<T>* gf;     // [n] forward segment products for this SEG
   const c2_t<T>* gb;     // [n] backward segment products for this SEG
   const c2_t<T>* ptab;   // [2][16][16] carry tables Pf, Pb for this SEG
-  // sub-step N (FIRST).  FP64 state: exp(-i dt V) (real time) or exp(-dt V)
-  // (imaginary time, real part only) as a per-point factor array fV, or for
-  // the separable harmonic trap as per-axis factors fx[i] fy[j] fz[k], and
-  // dtg = dt g for the nonlinear part.  FP32 state: the potential V (array) or
-  // vx[i] + vy[j] + vz[k], and dt, g: the phase angle is formed per point,
-  // because FP32-rounded factors would be applied identically every step and
-  // their |F| - 1 ~ 1e-7 would add up step after step.
+  // sub-step N (FIRST): the potential V (array) or vx[i] + vy[j] + vz[k], and
+  // dt, g: the phase angle is formed per point, because rounded factors would
+  // be applied identically every step and the rounding of |F| - 1 would add up
+  // step after step.  FP64 state, angles of 1/4 and more: the potential's part
+  // of the factor, exp(-i dt V) (real time) or exp(-dt V) (imaginary time, real
+  // part only), per point (fV) or for the separable harmonic trap per axis
+  // (fx[i] fy[j] fz[k]); dtg = dt g.
   const c2_t<T>* fV;
   const c2_t<T>* fx; const c2_t<T>* fy; const c2_t<T>* fz;
   T dtg;
@@ -116,7 +116,7 @@ struct Sweep2Args {
   int cdepth, cpts;
 };
 
-// Sub-step N at one point: p <- F exp(-i a) p (real time) or F exp(-a) p
+// Sub-step N at one point in factor form: p <- F exp(-i a) p (real time) or F exp(-a) p
 // (imaginary time), where F = exp(-i dt V) or exp(-dt V) is the precomputed
 // potential factor and a = dt g |p|^2.  The exponential of the nonlinear part
 // is its Taylor series: for |a| < 1/32 sin to a^7, cos to a^8, exp to a^7
@@ -261,6 +261,16 @@ __device__ __forceinline__ double2 phase_theta(double2 p, double th) {
     c = t2 * fma(t2, c, -1.0 / 2);
     return rot_apply<double>(p, s, c);
   }
+}
+
+// The FP64 sub-step N at one point with potential V: phase_theta below |th| =
+// 1/4 (every point of the workloads), else the factor form, whose cost does not
+// grow with the potential's part of the angle; F() gives the factor.
+template <bool IMAG, typename FacF>
+__device__ __forceinline__ double2 phase_f64(double2 p, double V, double dt, double g, FacF F) {
+  const double th = dt * fma(g, fma(p.x, p.x, p.y * p.y), V);
+  if (fabs(th) < 0.25) return phase_theta<IMAG>(p, th);
+  return phase_N<double, IMAG>(p, F(), dt * g);
 }
 
 // FP32 state: p <- exp(-i th) p or exp(-th) p with th = dt (V + g |p|^2)
@@ -585,8 +595,9 @@ __device__ __forceinline__ c2_t<T> half_phase(const Sweep2Args<T>& A, c2_t<T> w,
   if constexpr (is_df<T>::value) {
     return phase_df<IMAG>(w, A, q, i, j + A.geom.ny * kz, A.dtg);
   } else if constexpr (std::is_same<T, double>::value) {
-    const c2_t<T> F = A.fV ? A.fV[q] : fac_mul<T, IMAG>(A.fx[i], fac_mul<T, IMAG>(A.fy[j], A.fz[kz]));
-    return phase_N<T, IMAG>(w, F, A.dtg);
+    return phase_f64<IMAG>(w, A.V ? A.V[q] : A.vx[i] + (A.vy[j] + A.vz[kz]), A.dt, A.g, [&]() {
+      return A.fV ? A.fV[q] : fac_mul<T, IMAG>(A.fx[i], fac_mul<T, IMAG>(A.fy[j], A.fz[kz]));
+    });
   } else {
     return phase_direct<T, IMAG>(w, A.V ? A.V[q] : A.vx[i] + (A.vy[j] + A.vz[kz]), A.dt, A.g);
   }
@@ -755,39 +766,37 @@ __device__ __forceinline__ void tsweep_body(const Sweep2Args<T>& A, int L0, c2_t
   load_coefs<T>(A, sc, n);
   pdl_wait();  // the state and the norm sums are the previous kernels' output
   pdl_release();
-  constexpr bool kFactors = std::is_same<T, double>::value;  // FP64: precomputed potential factors
+  constexpr bool kF64 = std::is_same<T, double>::value;
   const int per_line = (n + 31) >> 5;  // n <= 512: at most 16 chunks
   const c2* in = A.src ? A.src : A.psi;
   const T* rin = reinterpret_cast<const T*>(in);  // RL
   const long lim = G.points();  // complex values (RL: reals) of the array
   // per-line part of the sub-step N (FIRST) of grid line Lg
-  auto line_factors = [&](int Lg, c2& fline, T& vline) {
-    fline = mk<T>(1, 0);
-    vline = T(0);
-    if (FIRST && Lg < G.nlines && !is_df<T>::value) {
-      if (kFactors && !A.fV) fline = fac_mul<T, IMAG>(A.fy[Lg % G.ny], A.fz[Lg / G.ny]);
-      if (!kFactors && !A.V) vline = A.vy[Lg % G.ny] + A.vz[Lg / G.ny];
-    }
+  auto line_part = [&](int Lg) -> T {
+    if (FIRST && Lg < G.nlines && !is_df<T>::value && !A.V) return A.vy[Lg % G.ny] + A.vz[Lg / G.ny];
+    return T(0);
   };
   // the factor scl and the sub-step N at interior point k of grid line Lg
-  auto apply_N = [&](c2 w, int Lg, int k, const c2& fline, T vline, T scl) -> c2 {
+  auto apply_N = [&](c2 w, int Lg, int k, T vline, T scl) -> c2 {
     const int gbase = Lg * G.nx;
     if constexpr (is_df<T>::value) {
       if (IMAG) { w.x *= scl; w.y *= scl; }
       return phase_df<IMAG>(w, A, gbase + k, k, Lg, A.dtg);
     } else {
       w.x *= scl; w.y *= scl;
-      if (kFactors) {
-        const c2 F = A.fV ? A.fV[gbase + k] : fac_mul<T, IMAG>(A.fx[k], fline);
-        return phase_N<T, IMAG>(w, F, A.dtg);
-      } else {
-        return phase_direct<T, IMAG>(w, A.V ? A.V[gbase + k] : A.vx[k] + vline, A.dt, A.g);
-      }
+      const T V = A.V ? A.V[gbase + k] : A.vx[k] + vline;
+      if constexpr (kF64)
+        return phase_f64<IMAG>(w, V, A.dt, A.g, [&]() {
+          return A.fV ? A.fV[gbase + k]
+                      : fac_mul<T, IMAG>(A.fx[k], fac_mul<T, IMAG>(A.fy[Lg % G.ny], A.fz[Lg / G.ny]));
+        });
+      else
+        return phase_direct<T, IMAG>(w, V, A.dt, A.g);
     }
   };
   // RL: N on one real value (as the complex path does on (x, 0))
-  auto apply_R = [&](T x, int Lg, int k, const c2& fline, T vline, T scl) -> T {
-    return apply_N(mk<T>(x, T(0)), Lg, k, fline, vline, scl).x;
+  auto apply_R = [&](T x, int Lg, int k, T vline, T scl) -> T {
+    return apply_N(mk<T>(x, T(0)), Lg, k, vline, scl).x;
   };
   // A pending renormalisation factor (imaginary time, after the first step)
   // is summed by warp 0 from the previous step's per-block norms while the
@@ -807,12 +816,7 @@ __device__ __forceinline__ void tsweep_body(const Sweep2Args<T>& A, int L0, c2_t
       if constexpr (RL) {
         const int La = 2 * (L0 + c), Lb = La + 1;
         const bool oka = line_ok, okb = line_ok && Lb < G.nlines;
-        c2 fa, fb;
-        T va, vb;
-        if (!pend) {
-          line_factors(La, fa, va);
-          line_factors(Lb, fb, vb);
-        }
+        const T va = pend ? T(0) : line_part(La), vb = pend ? T(0) : line_part(Lb);
         for (int q0 = 0; q0 < per_line; q0 += 4) {
           c2 v[4];
 #pragma unroll
@@ -828,17 +832,15 @@ __device__ __forceinline__ void tsweep_body(const Sweep2Args<T>& A, int L0, c2_t
             if (k >= n) break;
             c2 w = v[i];
             if (FIRST && !pend && k >= 1 && k <= M) {
-              if (oka) w.x = apply_R(w.x, La, k, fa, va, T(1));
-              if (okb) w.y = apply_R(w.y, Lb, k, fb, vb, T(1));
+              if (oka) w.x = apply_R(w.x, La, k, va, T(1));
+              if (okb) w.y = apply_R(w.y, Lb, k, vb, T(1));
             }
             if (GPE_CHECK(k < n && c < 32, 213)) tile[k * kTilePitch + c] = w;
           }
         }
       } else {
         const int gbase = (L0 + c) * G.nx;
-        c2 fline;
-        T vline;
-        if (!pend) line_factors(L0 + c, fline, vline);
+        const T vline = pend ? T(0) : line_part(L0 + c);
         for (int q0 = 0; q0 < per_line; q0 += 4) {
           c2 v[4];
 #pragma unroll
@@ -852,7 +854,7 @@ __device__ __forceinline__ void tsweep_body(const Sweep2Args<T>& A, int L0, c2_t
             const int k = (q0 + i) * 32 + lane;
             if (k >= n) break;
             c2 w = v[i];
-            if (FIRST && !pend && line_ok && k >= 1 && k <= M) w = apply_N(w, L0 + c, k, fline, vline, T(1));
+            if (FIRST && !pend && line_ok && k >= 1 && k <= M) w = apply_N(w, L0 + c, k, vline, T(1));
             if (GPE_CHECK(k < n && c < 32, 215)) tile[k * kTilePitch + c] = w;
           }
         }
@@ -866,24 +868,19 @@ __device__ __forceinline__ void tsweep_body(const Sweep2Args<T>& A, int L0, c2_t
       if constexpr (RL) {
         const int La = 2 * (L0 + c), Lb = La + 1;
         const bool okb = Lb < G.nlines;
-        c2 fa, fb;
-        T va, vb;
-        line_factors(La, fa, va);
-        line_factors(Lb, fb, vb);
+        const T va = line_part(La), vb = line_part(Lb);
         for (int k = lane; k < n; k += 32)
           if (k >= 1 && k <= M) {
             c2 w = tile[k * kTilePitch + c];
-            w.x = apply_R(w.x, La, k, fa, va, scl);
-            if (okb) w.y = apply_R(w.y, Lb, k, fb, vb, scl);
+            w.x = apply_R(w.x, La, k, va, scl);
+            if (okb) w.y = apply_R(w.y, Lb, k, vb, scl);
             tile[k * kTilePitch + c] = w;
           }
       } else {
-        c2 fline;
-        T vline;
-        line_factors(L0 + c, fline, vline);
+        const T vline = line_part(L0 + c);
         for (int k = lane; k < n; k += 32)
           if (k >= 1 && k <= M)
-            tile[k * kTilePitch + c] = apply_N(tile[k * kTilePitch + c], L0 + c, k, fline, vline, scl);
+            tile[k * kTilePitch + c] = apply_N(tile[k * kTilePitch + c], L0 + c, k, vline, scl);
       }
     }
   }
@@ -1119,14 +1116,9 @@ __device__ __forceinline__ void xsweep_body(const Sweep2Args<T>& A, int L, doubl
     c2* line = A.psi + base;
     const int k0 = 1 + lane * SEG;
     const int ta = L % G.ny, tb = L / G.ny;
-    constexpr bool kFactors = std::is_same<T, double>::value;  // FP64: precomputed potential factors
-    c2 fline = mk<T>(1, 0);
     T vline = T(0);
     const T scl = (T)pend;
-    if (FIRST && !is_df<T>::value) {
-      if (kFactors && A.fV == nullptr) fline = fac_mul<T, IMAG>(A.fy[ta], A.fz[tb]);
-      if (!kFactors && A.V == nullptr) vline = A.vy[ta] + A.vz[tb];
-    }
+    if (FIRST && !is_df<T>::value && A.V == nullptr) vline = A.vy[ta] + A.vz[tb];
     const c2* in = (A.src ? A.src : A.psi) + base;
     const long lim = G.points() - base;
     c2 p[SEG], e[SEG];
@@ -1141,12 +1133,13 @@ __device__ __forceinline__ void xsweep_body(const Sweep2Args<T>& A, int L, doubl
           v = phase_df<IMAG>(v, A, base + k, k, L, A.gw ? A.dtg * A.gw[k] : A.dtg);
         } else if constexpr (FIRST) {
           v.x *= scl; v.y *= scl;
-          if (kFactors) {
-            const c2 F = A.fV ? A.fV[base + k] : fac_mul<T, IMAG>(A.fx[k], fline);
-            v = phase_N<T, IMAG>(v, F, A.gw ? A.dtg * A.gw[k] : A.dtg);
-          } else {
-            v = phase_direct<T, IMAG>(v, A.V ? A.V[base + k] : A.vx[k] + vline, A.dt, A.gw ? A.g * A.gw[k] : A.g);
-          }
+          const T V = A.V ? A.V[base + k] : A.vx[k] + vline, gk = A.gw ? A.g * A.gw[k] : A.g;
+          if constexpr (std::is_same<T, double>::value)
+            v = phase_f64<IMAG>(v, V, A.dt, gk, [&]() {
+              return A.fV ? A.fV[base + k] : fac_mul<T, IMAG>(A.fx[k], fac_mul<T, IMAG>(A.fy[ta], A.fz[tb]));
+            });
+          else
+            v = phase_direct<T, IMAG>(v, V, A.dt, gk);
         }
       }
       p[j] = v;
@@ -1294,7 +1287,6 @@ __global__ void __launch_bounds__(512) psweep_kernel(Sweep2Args<T> A) {
   pdl_release();
   T scl = T(1);
   if (FIRST) scl = (T)pending_scale(A.parts_in, A.nparts_in, A.parts_wscale, red_smem);
-  constexpr bool kFactors = std::is_same<T, double>::value;
   static_assert(!is_df<T>::value, "the pipelined sweeps take FP32 and FP64 states");
   T tval = T(0);
   int it = 0;
@@ -1314,10 +1306,7 @@ __global__ void __launch_bounds__(512) psweep_kernel(Sweep2Args<T> A) {
       // sub-step N (and the pending renormalisation) on this thread's own points
       if (lane < nl) {
         const int L = L0 + lane;
-        c2 fline = mk<T>(1, 0);
-        T vline = T(0);
-        if (kFactors && !A.fV) fline = fac_mul<T, IMAG>(A.fy[L % G.ny], A.fz[L / G.ny]);
-        if (!kFactors && !A.V) vline = A.vy[L % G.ny] + A.vz[L / G.ny];
+        const T vline = A.V ? T(0) : A.vy[L % G.ny] + A.vz[L / G.ny];
         const int gb = L * G.nx;
 #pragma unroll
         for (int j = 0; j < SEG; ++j) {
@@ -1325,12 +1314,14 @@ __global__ void __launch_bounds__(512) psweep_kernel(Sweep2Args<T> A) {
           if (k <= M) {
             c2 w = at(k);
             w.x *= scl; w.y *= scl;
-            if (kFactors) {
-              const c2 F = A.fV ? A.fV[gb + k] : fac_mul<T, IMAG>(A.fx[k], fline);
-              w = phase_N<T, IMAG>(w, F, A.dtg);
-            } else {
-              w = phase_direct<T, IMAG>(w, A.V ? A.V[gb + k] : A.vx[k] + vline, A.dt, A.g);
-            }
+            const T V = A.V ? A.V[gb + k] : A.vx[k] + vline;
+            if constexpr (std::is_same<T, double>::value)
+              w = phase_f64<IMAG>(w, V, A.dt, A.g, [&]() {
+                return A.fV ? A.fV[gb + k]
+                            : fac_mul<T, IMAG>(A.fx[k], fac_mul<T, IMAG>(A.fy[L % G.ny], A.fz[L / G.ny]));
+              });
+            else
+              w = phase_direct<T, IMAG>(w, V, A.dt, A.g);
             at(k) = w;
           }
         }
@@ -1410,7 +1401,6 @@ __global__ void __launch_bounds__(256) strang_phase_kernel(Sweep2Args<T> A) {
   const unsigned cpl = (unsigned)(G.nx + 31) >> 5;  // chunks per x line
   const unsigned nchunks = cpl * (unsigned)G.nlines;
   const unsigned nwarps = gridDim.x * (blockDim.x >> 5);
-  constexpr bool kFactors = std::is_same<T, double>::value;
   T tacc = T(0);
   for (unsigned u0 = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * kStrangUnroll; u0 < nchunks;
        u0 += nwarps * kStrangUnroll) {
@@ -1435,12 +1425,14 @@ __global__ void __launch_bounds__(256) strang_phase_kernel(Sweep2Args<T> A) {
       c2 w = v[r];
       if constexpr (is_df<T>::value) {
         w = phase_df<IMAG>(w, A, q[r], i, L, A.gw ? A.dtg * A.gw[i] : A.dtg);
-      } else if constexpr (kFactors) {
-        const c2 F = A.fV ? A.fV[q[r]] : fac_mul<T, IMAG>(A.fx[i], fac_mul<T, IMAG>(A.fy[j], A.fz[k]));
-        w = phase_N<T, IMAG>(w, F, A.gw ? A.dtg * A.gw[i] : A.dtg);
       } else {
-        w = phase_direct<T, IMAG>(w, A.V ? A.V[q[r]] : A.vx[i] + (A.vy[j] + A.vz[k]), A.dt,
-                                  A.gw ? A.g * A.gw[i] : A.g);
+        const T V = A.V ? A.V[q[r]] : A.vx[i] + (A.vy[j] + A.vz[k]), gk = A.gw ? A.g * A.gw[i] : A.g;
+        if constexpr (std::is_same<T, double>::value)
+          w = phase_f64<IMAG>(w, V, A.dt, gk, [&]() {
+            return A.fV ? A.fV[q[r]] : fac_mul<T, IMAG>(A.fx[i], fac_mul<T, IMAG>(A.fy[j], A.fz[k]));
+          });
+        else
+          w = phase_direct<T, IMAG>(w, V, A.dt, gk);
       }
       A.psi[q[r]] = w;
       if (LAST) tacc += (A.w_axis[i] * (A.w_a[j] * A.w_b[k])) * (w.x * w.x + w.y * w.y);
