@@ -324,12 +324,12 @@ int upload_coefs_t(gp_handle* h) {
                     tabs.data() + (size_t)si * 512, n, kSegs[si], 1, tau, h->cdepth[mode][d][si], pts);
         h->cpts[mode][d][si] = carry_pts_class(pts);
       }
-      if (h->dim == 1) {
+      {
         // the points after which a product of the coefficients is below the threshold
         double amax = 0.0;
         for (int k = 1; k <= n - 2; ++k) amax = std::max({amax, std::abs(af[k]), std::abs(ab[k])});
         const double r = amax < 1.0 ? std::ceil(std::log(tau) / std::log(std::max(amax, 1e-300))) : (double)n;
-        h->line_reach[mode] = (long)std::min<double>(std::max(r, 1.0), (double)n);
+        h->axis_reach[mode][d] = (long)std::min<double>(std::max(r, 1.0), (double)n);
       }
       int rc = upload_c2<T>(h, h->coef[mode][d], all);
       if (rc) return rc;
@@ -785,9 +785,10 @@ int init_handle(gp_handle** out, int geom, int dim, const int n[3], const double
   h->tma_limit_ns = (unsigned long long)env_int("GPE_WAIT_LIMIT_MS", 1000) * 1000000ull;
   {
     // one norm sum per block of any last sweep: 32 lines per block (tiles and
-    // y/z sweeps), 4 (one-warp x lines), 128 (long lines), or a persistent grid
+    // y/z sweeps), 1 to 16 (tiles of few lines), 4 (one-warp x lines), 128 (long
+    // lines), or a persistent grid
     long maxparts = 152L * 32;
-    for (int d = 0; d < dim; ++d) maxparts = std::max(maxparts, h->np / h->n[d] / 4 + 1);
+    for (int d = 0; d < dim; ++d) maxparts = std::max(maxparts, h->np / h->n[d] + 1);
     for (int i = 0; i < 2; ++i)
       if ((rc = dev_alloc(h, (void**)&h->parts[i], (size_t)maxparts * sizeof(double)))) return bail(rc);
   }

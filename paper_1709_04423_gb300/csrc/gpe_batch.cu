@@ -23,6 +23,7 @@
 #include <type_traits>
 #include <vector>
 
+#include "gpe_flex.cuh"
 #include "gpe_internal.h"
 #include "gpe_obs.cuh"
 #include "gpe_sweep2.cuh"
@@ -87,16 +88,15 @@ __global__ void __launch_bounds__(512) batch_x_kernel(const BatchRun<T>* __restr
   tsweep_body<T, false, true, false, SEG>(A, it.L0, reinterpret_cast<c2_t<T>*>(bsmem_raw), cf, cb, red_smem);
 }
 
-// x lines whose shared-memory tile would not fit (FP64 and double-float,
-// n > 333): one warp per line, 4 lines per block; the item's L0 is the
-// block's first line.  The double-float body is held to 128 registers (four
-// blocks per SM): with the 234 it would take, 8 warps per SM left it
-// latency-bound (604 us per launch on the 64-run workload, ncu; the whole
-// double-float batch 7.29e9 -> 9.24e9 point-steps/s with the cap, 8.96e9 at
-// 80 registers).
-template <typename T, int SEG>
-__global__ void __launch_bounds__(128, std::is_same<T, df64>::value ? 4 : 1)
-    batch_xw_kernel(const BatchRun<T>* __restrict__ runs, const BatchItem* __restrict__ items, T dt) {
+// x lines whose 32-line tile would not fit in shared memory (FP64 and
+// double-float, n > 333): tiles of 8 lines (gpe_flex.cuh), segments of 32
+// points as the single-grid sweep's, 128 threads.
+constexpr int kBatchFlexLw = 3;
+
+template <typename T>
+__global__ void __launch_bounds__(128) batch_xf_kernel(const BatchRun<T>* __restrict__ runs,
+                                                       const BatchItem* __restrict__ items, T dt) {
+  extern __shared__ __align__(16) unsigned char bsmem_raw[];
   __shared__ double red_smem[32];
   const BatchItem it = items[blockIdx.x];
   const BatchRun<T>& R = runs[it.run];
@@ -113,6 +113,7 @@ __global__ void __launch_bounds__(128, std::is_same<T, df64>::value ? 4 : 1)
   A.alpha = R.coef[0];
   A.gf = R.coef[0] + R.nx;
   A.gb = R.coef[0] + 2 * R.nx;
+  A.ptab = R.ptab[0];
   A.cdepth = R.cdepth[0];
   A.cpts = R.cpts[0];
   A.fx = R.fx;
@@ -126,7 +127,8 @@ __global__ void __launch_bounds__(128, std::is_same<T, df64>::value ? 4 : 1)
   A.g = R.g;
   A.tfx = R.tfx;
   A.tfyz = R.tfy;
-  xsweep_body<T, false, true, false, SEG>(A, it.L0 + (threadIdx.x >> 5), red_smem);
+  const FlexTile F = flex_tile<T>(R.nx, kBatchFlexLw, 32);
+  flex_body<T, false, false, 32, true, false, false, false>(A, F, it.L0, reinterpret_cast<c2_t<T>*>(bsmem_raw), red_smem);
 }
 
 template <typename T, int SEG>
@@ -311,8 +313,8 @@ __global__ void __launch_bounds__(512) batch_persist_kernel(PersistArgs P) {
 // Segment-length classes: a line of n points goes to the first class whose
 // segment length gives at most 16 segments (the rule the single-grid handle
 // uses), so a run in a batch takes the same arithmetic as alone.  x lines
-// whose tile does not fit in shared memory form a fifth class, run one warp
-// per line (segment length = the smallest power of two >= (n-2)/32).
+// whose 32-line tile does not fit in shared memory form a fifth class, run in
+// tiles of 8 lines.
 constexpr int kNumClasses = 5;
 constexpr int kClassSegs[4] = {4, 8, 16, 32};
 constexpr int kBatchGraphSteps = 16;
@@ -336,7 +338,6 @@ struct gp_batch {
   void* items_d[2][5] = {{nullptr}};  // [axis][class]
   int nitems[2][5] = {{0}};
   int class_n[2][5] = {{0}};          // longest line of the class
-  int warp_seg = 16;                  // segment length of the warp-per-line class
   std::string launch_err;             // first failed launch of the current call
   // FP64 observables: per-run tables
   std::vector<void*> vd, cdx, wd;     // [nruns][2] device arrays, observables' arithmetic type
@@ -391,7 +392,7 @@ int b_upload(gp_batch* b, void* dst, const std::vector<T>& v) {
 
 bool x_tile_fits(int n, size_t esize) { return (36L * n + 512) * (long)esize <= 200L * 1024; }
 
-// class of a line of n points along axis a; class 4 = warp-per-line x lines
+// class of a line of n points along axis a; class 4 = x lines in tiles of few lines
 int class_of(int n, int a, size_t esize) {
   if (a == 0 && !x_tile_fits(n, esize)) return 4;
   const int M = n - 2;
@@ -400,20 +401,9 @@ int class_of(int n, int a, size_t esize) {
   return -1;
 }
 
-int warp_seg_of(int n) {
-  for (int s : {1, 2, 4, 8, 16})
-    if (32 * s >= n - 2) return s;
-  return 16;
-}
-
 template <typename T>
 int build_tables(gp_batch* b) {
   const int R = b->nruns;
-  // one segment length for every warp-per-line x line: enough for the longest
-  int nwarp = 0;
-  for (int r = 0; r < R; ++r)
-    if (class_of(b->n[2 * r], 0, b->esize) == 4) nwarp = std::max(nwarp, b->n[2 * r]);
-  b->warp_seg = nwarp ? warp_seg_of(nwarp) : 16;
   // coefficients: per run per axis 3n (alpha | gf | gb) + 512 carry tables
   std::vector<size_t> coff(2 * R), poff(2 * R);
   size_t ctot = 0;
@@ -442,7 +432,7 @@ int build_tables(gp_batch* b) {
       const double h = b->dx[2 * r + a];
       const AxisFactors f = thomas_factors(n, b->dt / (4.0 * h * h), false);
       const int cls = class_of(n, a, b->esize);
-      const int seg = cls == 4 ? b->warp_seg : kClassSegs[cls];
+      const int seg = cls == 4 ? 32 : kClassSegs[cls];
       std::vector<cd> gf, gb;
       segment_products(f.alpha, n, seg, gf, gb);
       cd tabs[512];
@@ -525,7 +515,7 @@ int build_tables(gp_batch* b) {
     for (int c = 0; c < kNumClasses; ++c) {
       std::vector<BatchItem> items;
       int nmax = 0;
-      const int step = c == 4 ? 4 : 32;         // lines per block
+      const int step = c == 4 ? 1 << kBatchFlexLw : 32;  // lines per block
       for (int r = 0; r < R; ++r) {
         const int n = b->n[2 * r + a];          // line length along axis a
         const int nl = b->n[2 * r + (1 - a)];   // number of lines
@@ -605,11 +595,13 @@ void enqueue_persistent(gp_batch* b, long nsteps) {
   count_launch();
 }
 
-template <typename T, int SEG>
-void launch_batch_warp(gp_batch* b) {
+template <typename T>
+void launch_batch_flex(gp_batch* b) {
   const auto* runs = (const BatchRun<T>*)b->runs_d;
   const auto* items = (const BatchItem*)b->items_d[0][4];
-  batch_xw_kernel<T, SEG><<<b->nitems[0][4], 128, 0, b->work>>>(runs, items, (T)b->dt);
+  const size_t smem = flex_elems(flex_tile<T>(b->class_n[0][4], kBatchFlexLw, 32)) * sizeof(c2_t<T>);
+  opt_in_smem((const void*)batch_xf_kernel<T>, smem);
+  batch_xf_kernel<T><<<b->nitems[0][4], 128, smem, b->work>>>(runs, items, (T)b->dt);
   count_launch();
 }
 
@@ -653,14 +645,7 @@ void enqueue_batch_step(gp_batch* b) {
         case 1: launch_batch_class<T, 8>(b, a, c); break;
         case 2: launch_batch_class<T, 16>(b, a, c); break;
         case 3: launch_batch_class<T, 32>(b, a, c); break;
-        default:
-          switch (b->warp_seg) {
-            case 1: launch_batch_warp<T, 1>(b); break;
-            case 2: launch_batch_warp<T, 2>(b); break;
-            case 4: launch_batch_warp<T, 4>(b); break;
-            case 8: launch_batch_warp<T, 8>(b); break;
-            default: launch_batch_warp<T, 16>(b); break;
-          }
+        default: launch_batch_flex<T>(b); break;
       }
     }
 }

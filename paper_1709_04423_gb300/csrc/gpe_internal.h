@@ -107,8 +107,8 @@ struct gp_handle {
   // per mode, axis and segment length: the segment carries' reach (Sweep2Args cdepth, cpts)
   int cdepth[gpe::NUM_MODES][3][gpe::kNumSegs] = {};
   int cpts[gpe::NUM_MODES][3][gpe::kNumSegs] = {};
-  // 1d grids: points over which a carry falls below the precision's threshold
-  long line_reach[gpe::NUM_MODES] = {0};
+  // per mode and axis: points over which a carry falls below the precision's threshold
+  long axis_reach[gpe::NUM_MODES][3] = {};
   // circular / axial traps (geom 2): per mode, the rho axis' backward
   // coefficients, forward right-hand-side factors and stencil factors
   // (vab, vbf, vh of Sweep2Args; 3 n[0] complex values)

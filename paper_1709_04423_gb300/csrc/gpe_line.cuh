@@ -517,7 +517,7 @@ int run_line_t(gp_handle* h, bool imag, long nsteps) {
   fill(L.a, h->strang && imag);
   fill(L.h, h->strang);
   // levels: 2^levels threads of S points reach as far as the coefficients do; depth: the same in warps
-  const long reach = h->line_reach[mode];
+  const long reach = h->axis_reach[mode][0];
   while (L.levels < 5 && ((1L << L.levels) - 1) * plan.S < reach) ++L.levels;
   L.depth = (int)std::max<long>(1, std::min<long>(kLineMaxWarps, (reach + 32L * plan.S - 1) / (32L * plan.S)));
   L.close_each = h->strang && imag;

@@ -12,6 +12,7 @@
 #include <cstring>
 
 #include "gpe_adjoint.cuh"
+#include "gpe_flex.cuh"
 #include "gpe_internal.h"
 #include "gpe_obs.cuh"
 #include "gpe_sweep.cuh"
@@ -24,6 +25,7 @@ namespace gpe {
 
 constexpr int kLegacyThreads = 128;
 constexpr int kXWarps = 4;
+constexpr unsigned kFoldParts = 4096;  // more norm sums than this are folded before the next step reads them
 constexpr int kGraphSteps = 16;  // even: keeps the renormalisation-slot parity
 
 inline LineGeom geom_of(const gp_handle* h, int axis) {
@@ -380,6 +382,45 @@ inline bool strang_close_fused(const gp_handle* h, bool imag) {
   return imag && h->strang && h->dim > 1 && h->seg_c > 0 && !h->pipe_c;
 }
 
+// The tiles of few lines (gpe_flex.cuh) of the sweep along axis d, or threads =
+// 0 where another kernel takes it.  They take lines of more than 514 points
+// (without them a thread walks a whole line: 1000 x 1000 FP64 imaginary time
+// 2840 -> 150 us per step), x lines for which no 32-line tile was chosen, and
+// grids with few 32-line tiles (us per sweep, 32-line tiles -> these):
+//  * FP64, fewer than 96 tiles: 257 x 201 real x 111.6 -> 21.6, y 44.4 -> 16.6;
+//    64^3 (128 tiles) would lose, x 25.3 -> 29.0, z 15.0 -> 17.6;
+//  * FP32 x, fewer than 64 tiles: 257 x 201 10.4 -> 7.9, 512^2 imaginary 18.9 ->
+//    9.2; 64^3 would lose, 5.0 -> 6.5;
+//  * FP32 y/z, fewer than 64 tiles of 32-point segments (lines over 258 points):
+//    512^2 imaginary 11.7 -> 5.2; 257 x 201 (16-point ones) would lose, 4.2 -> 5.4,
+//    to the staging through shared memory;
+//  * double-float x, fewer than 64 tiles: 257 x 201 37.8 -> 29.9; y would lose,
+//    19.0 -> 20.5.
+// The plan picks the segments' length on 2d grids in imaginary time and on axial
+// ones; elsewhere they keep the handle's: Cartesian 2d real-time runs agree bit
+// for bit with the same run in a batch, and the shapes of a 3d grid with each other.
+template <typename T>
+FlexPlan flex_sweep(const gp_handle* h, bool imag, int d, int seg) {
+  const int n = axis_len(h, d);
+  const long nlines = h->np / n;
+  if (h->dim == 1 || h->real_mode) return FlexPlan();
+  const long reach = h->axis_reach[imag ? MODE_IMAG : MODE_REAL][d];
+  if (seg > 0) {
+    if (d == 0 ? h->pipe_x || h->tma_x : h->pipe_c || h->tma_c) return FlexPlan();
+    if (d < 2 && xy_fused(h)) return FlexPlan();
+    if (d > 0 || h->tile_x) {
+      const long tiles = (nlines + 31) / 32;
+      if (tiles >= (std::is_same<T, double>::value ? 96 : 64)) return FlexPlan();
+      if (d > 0 && (is_df<T>::value || (std::is_same<T, float>::value && seg < 32))) return FlexPlan();
+    }
+    if (h->dim == 2 && (imag || h->geom == 2)) seg = 0;
+    else if (d == 0 && !h->tile_x) seg = tile_seg(n - 2);
+  } else if (!imag) {
+    seg = tile_seg(n - 2);  // (0 for the lines over 514 points)
+  }
+  return flex_plan<T>(n, nlines, seg, d == 0, reach);
+}
+
 // Returns whether the sweep applied the step's closing N(dt/2).
 template <typename T>
 bool enqueue_sweep(gp_handle* h, bool imag, NormSlots ns, int d, const void* src = nullptr, bool half_open = true) {
@@ -394,13 +435,14 @@ bool enqueue_sweep(gp_handle* h, bool imag, NormSlots ns, int d, const void* src
   unsigned blocks = 0;
   const bool fuse_xy = xy_fused(h) && src == nullptr && (d == 0 || d == 1);
   if (fuse_xy && d == 1) return false;  // done by the fused x + y kernel
-  if (seg > 0) {
+  const FlexPlan flex = flex_sweep<T>(h, imag, d, seg);
+  if (seg > 0 || flex.threads > 0) {
     Sweep2Args<T> a;
     std::memset(&a, 0, sizeof(a));
     a.psi = (c2_t<T>*)h->psi;
     a.src = d == 0 ? (const c2_t<T>*)src : nullptr;
     a.geom = geom_of(h, d);
-    const int si = seg_index(seg);
+    const int si = seg_index(flex.threads > 0 ? flex.seg : seg);
     a.alpha = coef_ptr<T>(h, mode, d, 0);
     a.gf = coef_ptr<T>(h, mode, d, 1 + 2 * si);
     a.gb = coef_ptr<T>(h, mode, d, 2 + 2 * si);
@@ -424,6 +466,17 @@ bool enqueue_sweep(gp_handle* h, bool imag, NormSlots ns, int d, const void* src
       a.vh = cv + 2 * h->n[0];
     }
     bool done = false;
+    if (flex.threads > 0) {
+      run_flex<T>(a, flex, imag, write, fuse_close, var, h->work, h->pdl_now);
+      count_launch();
+      blocks = flex.blocks;
+      if (write && blocks > kFoldParts) {
+        launch_k(h->pdl_now, fold_parts_kernel, dim3(1), dim3(1024), 0, h->work, parts_out, (int)blocks);
+        count_launch();
+        blocks = 1;
+      }
+      done = true;
+    }
     if constexpr (std::is_same<T, float>::value) {
       if (fuse_xy) {  // d == 0: the y axis' coefficients beside the x sweep's arguments
         Sweep2Args<float> ay;
@@ -440,7 +493,8 @@ bool enqueue_sweep(gp_handle* h, bool imag, NormSlots ns, int d, const void* src
         done = true;
       }
     }
-    if (var) {
+    if (done) {
+    } else if (var) {
       if (h->tile_x) {  // axial trap: x is not the last axis
         blocks = imag ? launch_t_seg<T, true, true, false, false, true>(seg, a, h->work, h->pdl_now)
                       : launch_t_seg<T, false, true, false, false, true>(seg, a, h->work, h->pdl_now);

@@ -265,9 +265,13 @@ __device__ __forceinline__ double2 phase_theta(double2 p, double th) {
 
 // The FP64 sub-step N at one point with potential V: phase_theta below |th| =
 // 1/4 (every point of the workloads), else the factor form, whose cost does not
-// grow with the potential's part of the angle; F() gives the factor.
-template <bool IMAG, typename FacF>
+// grow with the potential's part of the angle; F() gives the factor.  ANY: in
+// imaginary time too; else imaginary time takes the factor form throughout --
+// its 15 operations do not depend on the angle, where the whole angle's longer
+// series above 1/32 takes 18 (64^3 at dt = 5e-4: x sweep 25.3 against 28.7 us).
+template <bool IMAG, bool ANY = false, typename FacF>
 __device__ __forceinline__ double2 phase_f64(double2 p, double V, double dt, double g, FacF F) {
+  if constexpr (IMAG && !ANY) return phase_N<double, IMAG>(p, F(), dt * g);
   const double th = dt * fma(g, fma(p.x, p.x, p.y * p.y), V);
   if (fabs(th) < 0.25) return phase_theta<IMAG>(p, th);
   return phase_N<double, IMAG>(p, F(), dt * g);
@@ -772,31 +776,39 @@ __device__ __forceinline__ void tsweep_body(const Sweep2Args<T>& A, int L0, c2_t
   const T* rin = reinterpret_cast<const T*>(in);  // RL
   const long lim = G.points();  // complex values (RL: reals) of the array
   // per-line part of the sub-step N (FIRST) of grid line Lg
-  auto line_part = [&](int Lg) -> T {
-    if (FIRST && Lg < G.nlines && !is_df<T>::value && !A.V) return A.vy[Lg % G.ny] + A.vz[Lg / G.ny];
-    return T(0);
+  // (FP64 imaginary time works with factors, see phase_f64, the others with angles)
+  constexpr bool kFac = kF64 && IMAG;
+  auto line_part = [&](int Lg, c2& fline, T& vline) {
+    fline = mk<T>(1, 0);
+    vline = T(0);
+    if (FIRST && Lg < G.nlines && !is_df<T>::value) {
+      if (kFac && !A.fV) fline = fac_mul<T, IMAG>(A.fy[Lg % G.ny], A.fz[Lg / G.ny]);
+      if (!kFac && !A.V) vline = A.vy[Lg % G.ny] + A.vz[Lg / G.ny];
+    }
   };
   // the factor scl and the sub-step N at interior point k of grid line Lg
-  auto apply_N = [&](c2 w, int Lg, int k, T vline, T scl) -> c2 {
+  auto apply_N = [&](c2 w, int Lg, int k, const c2& fline, T vline, T scl) -> c2 {
     const int gbase = Lg * G.nx;
     if constexpr (is_df<T>::value) {
       if (IMAG) { w.x *= scl; w.y *= scl; }
       return phase_df<IMAG>(w, A, gbase + k, k, Lg, A.dtg);
     } else {
       w.x *= scl; w.y *= scl;
-      const T V = A.V ? A.V[gbase + k] : A.vx[k] + vline;
-      if constexpr (kF64)
-        return phase_f64<IMAG>(w, V, A.dt, A.g, [&]() {
+      if constexpr (kFac) {
+        return phase_N<T, IMAG>(w, A.fV ? A.fV[gbase + k] : fac_mul<T, IMAG>(A.fx[k], fline), A.dtg);
+      } else if constexpr (kF64) {
+        return phase_f64<IMAG>(w, A.V ? A.V[gbase + k] : A.vx[k] + vline, A.dt, A.g, [&]() {
           return A.fV ? A.fV[gbase + k]
                       : fac_mul<T, IMAG>(A.fx[k], fac_mul<T, IMAG>(A.fy[Lg % G.ny], A.fz[Lg / G.ny]));
         });
-      else
-        return phase_direct<T, IMAG>(w, V, A.dt, A.g);
+      } else {
+        return phase_direct<T, IMAG>(w, A.V ? A.V[gbase + k] : A.vx[k] + vline, A.dt, A.g);
+      }
     }
   };
   // RL: N on one real value (as the complex path does on (x, 0))
-  auto apply_R = [&](T x, int Lg, int k, T vline, T scl) -> T {
-    return apply_N(mk<T>(x, T(0)), Lg, k, vline, scl).x;
+  auto apply_R = [&](T x, int Lg, int k, const c2& fline, T vline, T scl) -> T {
+    return apply_N(mk<T>(x, T(0)), Lg, k, fline, vline, scl).x;
   };
   // A pending renormalisation factor (imaginary time, after the first step)
   // is summed by warp 0 from the previous step's per-block norms while the
@@ -816,7 +828,12 @@ __device__ __forceinline__ void tsweep_body(const Sweep2Args<T>& A, int L0, c2_t
       if constexpr (RL) {
         const int La = 2 * (L0 + c), Lb = La + 1;
         const bool oka = line_ok, okb = line_ok && Lb < G.nlines;
-        const T va = pend ? T(0) : line_part(La), vb = pend ? T(0) : line_part(Lb);
+        c2 fa, fb;
+        T va, vb;
+        if (!pend) {
+          line_part(La, fa, va);
+          line_part(Lb, fb, vb);
+        }
         for (int q0 = 0; q0 < per_line; q0 += 4) {
           c2 v[4];
 #pragma unroll
@@ -832,15 +849,17 @@ __device__ __forceinline__ void tsweep_body(const Sweep2Args<T>& A, int L0, c2_t
             if (k >= n) break;
             c2 w = v[i];
             if (FIRST && !pend && k >= 1 && k <= M) {
-              if (oka) w.x = apply_R(w.x, La, k, va, T(1));
-              if (okb) w.y = apply_R(w.y, Lb, k, vb, T(1));
+              if (oka) w.x = apply_R(w.x, La, k, fa, va, T(1));
+              if (okb) w.y = apply_R(w.y, Lb, k, fb, vb, T(1));
             }
             if (GPE_CHECK(k < n && c < 32, 213)) tile[k * kTilePitch + c] = w;
           }
         }
       } else {
         const int gbase = (L0 + c) * G.nx;
-        const T vline = pend ? T(0) : line_part(L0 + c);
+        c2 fline;
+        T vline;
+        if (!pend) line_part(L0 + c, fline, vline);
         for (int q0 = 0; q0 < per_line; q0 += 4) {
           c2 v[4];
 #pragma unroll
@@ -854,7 +873,7 @@ __device__ __forceinline__ void tsweep_body(const Sweep2Args<T>& A, int L0, c2_t
             const int k = (q0 + i) * 32 + lane;
             if (k >= n) break;
             c2 w = v[i];
-            if (FIRST && !pend && line_ok && k >= 1 && k <= M) w = apply_N(w, L0 + c, k, vline, T(1));
+            if (FIRST && !pend && line_ok && k >= 1 && k <= M) w = apply_N(w, L0 + c, k, fline, vline, T(1));
             if (GPE_CHECK(k < n && c < 32, 215)) tile[k * kTilePitch + c] = w;
           }
         }
@@ -868,19 +887,24 @@ __device__ __forceinline__ void tsweep_body(const Sweep2Args<T>& A, int L0, c2_t
       if constexpr (RL) {
         const int La = 2 * (L0 + c), Lb = La + 1;
         const bool okb = Lb < G.nlines;
-        const T va = line_part(La), vb = line_part(Lb);
+        c2 fa, fb;
+        T va, vb;
+        line_part(La, fa, va);
+        line_part(Lb, fb, vb);
         for (int k = lane; k < n; k += 32)
           if (k >= 1 && k <= M) {
             c2 w = tile[k * kTilePitch + c];
-            w.x = apply_R(w.x, La, k, va, scl);
-            if (okb) w.y = apply_R(w.y, Lb, k, vb, scl);
+            w.x = apply_R(w.x, La, k, fa, va, scl);
+            if (okb) w.y = apply_R(w.y, Lb, k, fb, vb, scl);
             tile[k * kTilePitch + c] = w;
           }
       } else {
-        const T vline = line_part(L0 + c);
+        c2 fline;
+        T vline;
+        line_part(L0 + c, fline, vline);
         for (int k = lane; k < n; k += 32)
           if (k >= 1 && k <= M)
-            tile[k * kTilePitch + c] = apply_N(tile[k * kTilePitch + c], L0 + c, k, vline, scl);
+            tile[k * kTilePitch + c] = apply_N(tile[k * kTilePitch + c], L0 + c, k, fline, vline, scl);
       }
     }
   }
