@@ -54,7 +54,7 @@ template <typename T> __device__ __forceinline__ c2_t<T> mk(T x, T y) { c2_t<T> 
 // rounding does not depend on how the compiler contracts the expression in a
 // given kernel (the batched and the single-grid kernels then agree bit for bit).
 template <typename T> __device__ __forceinline__ c2_t<T> cmul(c2_t<T> a, c2_t<T> b) {
-  if constexpr (is_df<T>::value) return mk<T>(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
+  if constexpr (is_df<T>::value) return mk<T>(dfl::df_dot2(a.x, b.x, a.y, b.y), dfl::df_dot2(a.x, b.y, -a.y, b.x));
   else return mk<T>(fma(a.x, b.x, -(a.y * b.y)), fma(a.x, b.y, a.y * b.x));
 }
 

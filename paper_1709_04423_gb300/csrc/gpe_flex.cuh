@@ -50,8 +50,8 @@ __host__ __device__ inline FlexTile flex_tile(int n, int lw, int seg) {
 // Shared memory of a tile, in elements: the lines, then the two carry arrays.
 inline size_t flex_elems(const FlexTile& t) { return ((size_t)t.P + 2 * (size_t)t.nseg) << t.lw; }
 
-// The values a solving thread works on: whole complex points, or (SPLIT, FP64)
-// one component each, neighbouring lanes holding the two of a point.  One warp
+// The values a solving thread works on: whole complex points, or (SPLIT, FP64
+// and double-float) one component each, neighbouring lanes holding the two of a point.  One warp
 // gets an FP64 result every 64 clocks whatever its active lanes, four warps
 // of an SM together one every 19 (measured with chains of FMAs), so on grids
 // with too few lines to keep four warps per SM busy a thread per component
@@ -67,7 +67,7 @@ struct FlexOps {
   static __device__ __forceinline__ void set(c2_t<T>& d, int, const V& v) { d = v; }
   static __device__ __forceinline__ V other(const V& v) { return v; }
   static __device__ __forceinline__ V lap_add(const V& q, const V& l, const V& r, const V& p) {
-    return mk<T>(q.x + neg_lap(l.x, r.x, p.x), q.y + neg_lap(l.y, r.y, p.y));
+    return mk<T>(gpe::lap_add(q.x, l.x, r.x, p.x), gpe::lap_add(q.y, l.y, r.y, p.y));
   }
   static __device__ __forceinline__ V lapv(const V& l, const V& r, const V& p, const c2_t<T>& h) {
     return mk<T>(gpe::lapv(l.x, r.x, p.x, h.x, h.y), gpe::lapv(l.y, r.y, p.y, h.x, h.y));
@@ -83,45 +83,45 @@ struct FlexOps {
   static __device__ __forceinline__ T sq(const V& u) { return u.x * u.x + u.y * u.y; }
 };
 
-template <bool IMAG>
-struct FlexOps<double, IMAG, true> {
-  using V = double;
-  static __device__ __forceinline__ double flip(double v, int comp) {  // -v for the real part's thread
-    return comp ? v : -v;
+template <typename T, bool IMAG>
+struct FlexOps<T, IMAG, true> {
+  using V = T;
+  static __device__ __forceinline__ T flip(T v, int comp) { return comp ? v : -v; }  // -v for the real part's thread
+  static __device__ __forceinline__ T zero() { return T(0); }
+  static __device__ __forceinline__ T part(const c2_t<T>& p, int comp) { return reinterpret_cast<const T*>(&p)[comp]; }
+  static __device__ __forceinline__ c2_t<T> full(T v, int comp) {
+    const T o = shfl_xor_t(v, 1);
+    return comp ? mk<T>(o, v) : mk<T>(v, o);
   }
-  static __device__ __forceinline__ double zero() { return 0.0; }
-  static __device__ __forceinline__ double part(const double2& p, int comp) {
-    return reinterpret_cast<const double*>(&p)[comp];
+  static __device__ __forceinline__ void set(c2_t<T>& d, int comp, T v) { reinterpret_cast<T*>(&d)[comp] = v; }
+  static __device__ __forceinline__ T other(T v) {
+    if constexpr (IMAG) return v;
+    else return shfl_xor_t(v, 1);
   }
-  static __device__ __forceinline__ double2 full(double v, int comp) {
-    const double o = __shfl_xor_sync(0xffffffffu, v, 1);
-    return comp ? make_double2(o, v) : make_double2(v, o);
+  static __device__ __forceinline__ T lap_add(T q, T l, T r, T p) { return gpe::lap_add(q, l, r, p); }
+  static __device__ __forceinline__ T lapv(T l, T r, T p, const c2_t<T>& h) { return gpe::lapv(l, r, p, h.x, h.y); }
+  static __device__ __forceinline__ T mul(const c2_t<T>& a, T b, int comp) {
+    if constexpr (IMAG) return a.x * b;
+    else if constexpr (is_df<T>::value) return dfl::df_dot2(a.x, b, flip(-a.y, comp), other(b));
+    else return ::fma(a.x, b, flip(a.y, comp) * other(b));
   }
-  static __device__ __forceinline__ void set(double2& d, int comp, double v) {
-    reinterpret_cast<double*>(&d)[comp] = v;
+  static __device__ __forceinline__ T fma_pair(const c2_t<T>& a, T b, T o, T c, int comp) {
+    if constexpr (is_df<T>::value) {
+      if constexpr (IMAG) return dfl::fma(a.x, b, c);
+      else return dfl::df_dot2_add(a.x, b, flip(-a.y, comp), o, c);
+    } else {
+      if constexpr (IMAG) return ::fma(a.x, b, c);
+      else return ::fma(a.x, b, ::fma(flip(a.y, comp), o, c));
+    }
   }
-  static __device__ __forceinline__ double other(double v) {
-    return IMAG ? v : __shfl_xor_sync(0xffffffffu, v, 1);
-  }
-  static __device__ __forceinline__ double lap_add(double q, double l, double r, double p) {
-    return q + neg_lap(l, r, p);
-  }
-  static __device__ __forceinline__ double lapv(double l, double r, double p, const double2& h) {
-    return gpe::lapv(l, r, p, h.x, h.y);
-  }
-  static __device__ __forceinline__ double mul(const double2& a, double b, int comp) {
-    if (IMAG) return a.x * b;
-    return ::fma(a.x, b, flip(a.y, comp) * other(b));
-  }
-  static __device__ __forceinline__ double fma_pair(const double2& a, double b, double o, double c, int comp) {
-    if (IMAG) return ::fma(a.x, b, c);
-    return ::fma(a.x, b, ::fma(flip(a.y, comp), o, c));
-  }
-  static __device__ __forceinline__ double fma(const double2& a, double b, double c, int comp) {
+  static __device__ __forceinline__ T fma(const c2_t<T>& a, T b, T c, int comp) {
     return fma_pair(a, b, other(b), c, comp);
   }
-  static __device__ __forceinline__ double sub2(double p, double z) { return ::fma(-2.0, z, p); }
-  static __device__ __forceinline__ double sq(double u) { return u * u; }
+  static __device__ __forceinline__ T sub2(T p, T z) {
+    if constexpr (is_df<T>::value) return dfl::df_sub2(p, z);
+    else return ::fma(T(-2), z, p);
+  }
+  static __device__ __forceinline__ T sq(T u) { return u * u; }
 };
 
 // Lines L0 .. L0 + W - 1 of the grid described by A.  AXIS0: x lines, with
@@ -405,20 +405,20 @@ struct FlexPlan {
   FlexTile t = {0, 0, 0, 0};
   int seg = 0, threads = 0;
   unsigned blocks = 0;
-  bool split = false;  // FP64: a thread per component
+  bool split = false;  // FP64 and double-float: a thread per component
 };
 
 // The tile is the widest of 16 lines and fewer that gives one and a half
 // blocks per SM.  Where the solving warps would still be fewer than four per SM
-// (an SM's FP64 rate needs four; FP32 and double-float chains only get shorter),
-// free segments are halved down to 8 points and FP64 takes a thread per component.
+// (an SM's FP64 rate needs four; the other chains only get shorter), free segments
+// are halved down to 8 points and FP64 and double-float take a thread per component.
 template <typename T>
 FlexPlan flex_plan(int n, long nlines, int seg, bool axis0, long reach) {
   FlexPlan p;
   const int M = n - 2;
   const int lmin = axis0 ? 1 : sizeof(c2_t<T>) == 8 ? 2 : 1;
   const bool few = nlines * ((M + 15) / 16) < 32L * 4 * 152;
-  p.split = few && std::is_same<T, double>::value;
+  p.split = few && !std::is_same<T, float>::value;
   for (int lw = 4; lw >= 0; --lw) {
     const int ls = lw + (p.split ? 1 : 0);
     p.seg = seg;
@@ -441,7 +441,7 @@ FlexPlan flex_plan(int n, long nlines, int seg, bool axis0, long reach) {
 template <typename T, bool IMAG, bool LAST, int SEG, bool AXIS0, bool VAR, bool CLOSE>
 void launch_flex(const Sweep2Args<T>& a, const FlexPlan& p, cudaStream_t s, bool pdl) {
   auto kern = flex_kernel<T, IMAG, LAST, SEG, AXIS0, VAR, CLOSE, false>;
-  if constexpr (std::is_same<T, double>::value)
+  if constexpr (!std::is_same<T, float>::value)
     if (p.split) kern = flex_kernel<T, IMAG, LAST, SEG, AXIS0, VAR, CLOSE, true>;
   opt_in_smem((const void*)kern, 200 * 1024);
   launch_k(pdl, kern, dim3(p.blocks), dim3(p.threads), flex_elems(p.t) * sizeof(c2_t<T>), s, a, p.t);

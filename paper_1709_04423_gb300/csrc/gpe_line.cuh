@@ -277,8 +277,9 @@ __global__ void __launch_bounds__(kLineMaxThreads) line_steps_kernel(const __gri
           const c2 v = cf_mul<T, IMAG>(bf[j], lv);
           prev = j == 0 ? v : cf_fma<T, IMAG>(al[j], prev, v);
         } else {
-          c2 v = mk<T>(neg_lap(left.x, right.x, p[j].x), neg_lap(left.y, right.y, p[j].y));
-          if (j > 0) v = mk<T>(prev.x + v.x, prev.y + v.y);
+          const c2 v = j == 0 ? mk<T>(neg_lap(left.x, right.x, p[j].x), neg_lap(left.y, right.y, p[j].y))
+                              : mk<T>(lap_add(prev.x, left.x, right.x, p[j].x),
+                                      lap_add(prev.y, left.y, right.y, p[j].y));
           prev = cf_mul<T, IMAG>(al[j], v);
         }
         e[j] = prev;

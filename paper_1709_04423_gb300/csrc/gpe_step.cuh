@@ -411,7 +411,7 @@ FlexPlan flex_sweep(const gp_handle* h, bool imag, int d, int seg) {
     if (d > 0 || h->tile_x) {
       const long tiles = (nlines + 31) / 32;
       if (tiles >= (std::is_same<T, double>::value ? 96 : 64)) return FlexPlan();
-      if (d > 0 && (is_df<T>::value || (std::is_same<T, float>::value && seg < 32))) return FlexPlan();
+      if (d > 0 && std::is_same<T, float>::value && seg < 32) return FlexPlan();
     }
     if (h->dim == 2 && (imag || h->geom == 2)) seg = 0;
     else if (d == 0 && !h->tile_x) seg = tile_seg(n - 2);

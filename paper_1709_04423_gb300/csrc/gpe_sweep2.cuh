@@ -319,7 +319,7 @@ __device__ __forceinline__ c2_t<T> phase_direct(c2_t<T> p, T V, T dt, T g) {
 template <bool IMAG>
 __device__ __forceinline__ df64x2 phase_df(df64x2 p, const Sweep2Args<df64>& A, long gidx, int k, int L,
                                            df64 dtg) {
-  const df64 a = dtg * (p.x * p.x + p.y * p.y);
+  const df64 a = dtg * dfl::df_dot2(p.x, p.x, -p.y, p.y);
   if (IMAG) {
     df64 e;
     if (fabsf(a.hi) < 0.125f) {
@@ -328,11 +328,11 @@ __device__ __forceinline__ df64x2 phase_df(df64x2 p, const Sweep2Args<df64>& A, 
       const float te = 1.0f / 720 + mf * (1.0f / 5040 + mf * (1.0f / 40320 + mf * (1.0f / 362880 + mf * (1.0f / 3628800))));
       constexpr df64 c5(1.0 / 120), c4(1.0 / 24), c3(1.0 / 6), c2(0.5), c1(1.0);
       e = df_mulf(m, te) + c5;
-      e = m * e + c4;
-      e = m * e + c3;
-      e = m * e + c2;
-      e = m * e + c1;
-      e = m * e + c1;
+      e = fma(m, e, c4);
+      e = fma(m, e, c3);
+      e = fma(m, e, c2);
+      e = fma(m, e, c1);
+      e = fma(m, e, c1);
     } else {
       e = df64(::exp(-(double)a));
     }
@@ -355,12 +355,12 @@ __device__ __forceinline__ df64x2 phase_df(df64x2 p, const Sweep2Args<df64>& A, 
       const float tc = -1.0f / 720 + q * (1.0f / 40320 + q * (-1.0f / 3628800 + q * (1.0f / 479001600)));
       constexpr df64 s2(1.0 / 120), s1(-1.0 / 6), c2(1.0 / 24), c1(-0.5), one(1.0);
       df64 S = df_mulf(a2, ts) + s2;
-      S = a2 * S + s1;
-      S = a2 * S + one;
+      S = fma(a2, S, s1);
+      S = fma(a2, S, one);
       sn = a * S;
       df64 C = df_mulf(a2, tc) + c2;
-      C = a2 * C + c1;
-      cs = a2 * C + one;
+      C = fma(a2, C, c1);
+      cs = fma(a2, C, one);
     } else {
       double sd, cd;
       ::sincos((double)a, &sd, &cd);
@@ -368,7 +368,7 @@ __device__ __forceinline__ df64x2 phase_df(df64x2 p, const Sweep2Args<df64>& A, 
       cs = df64(cd);
     }
     // exp(-i a) p = (cs px + sn py) + i (cs py - sn px)
-    p = df64x2{cs * p.x + sn * p.y, cs * p.y - sn * p.x};
+    p = df64x2{dfl::df_dot2(cs, p.x, -sn, p.y), dfl::df_dot2(cs, p.y, sn, p.x)};
     auto cmul_tf = [](const tf3c& F, df64x2 v) {
       // (Fr + i Fi)(vx + i vy) = (Fr vx - Fi vy) + i (Fr vy - Fi (-vx))
       return df64x2{tf_dot2(F.re, v.x, F.im, v.y), tf_dot2(F.re, v.y, F.im, -v.x)};
@@ -400,7 +400,9 @@ __device__ __forceinline__ c2_t<T> cf_mul(c2_t<T> a, c2_t<T> b) {
 template <typename T, bool IMAG>
 __device__ __forceinline__ c2_t<T> cf_fma(c2_t<T> a, c2_t<T> b, c2_t<T> c) {
   if (IMAG) return mk<T>(fma(a.x, b.x, c.x), fma(a.x, b.y, c.y));
-  return mk<T>(fma(a.x, b.x, fma(-a.y, b.y, c.x)), fma(a.x, b.y, fma(a.y, b.x, c.y)));
+  if constexpr (is_df<T>::value)
+    return mk<T>(dfl::df_dot2_add(a.x, b.x, a.y, b.y, c.x), dfl::df_dot2_add(a.x, b.y, -a.y, b.x, c.y));
+  else return mk<T>(fma(a.x, b.x, fma(-a.y, b.y, c.x)), fma(a.x, b.y, fma(a.y, b.x, c.y)));
 }
 // coefficient product a * b (both coefficients)
 template <typename T, bool IMAG>
@@ -422,14 +424,20 @@ __device__ __forceinline__ c2_t<T> shfl_down2(c2_t<T> v, int o) {
 // depend on the recurrence (exactly half of 4 p - 2 (l + r))
 template <typename T>
 __device__ __forceinline__ T neg_lap(T l, T r, T p) {
-  if constexpr (is_df<T>::value) return df_scale(p, 2.f) - (l + r);
+  if constexpr (is_df<T>::value) return dfl::df_lap(l, r, p);
   else return fma(T(2), p, -(l + r));
+}
+// q + 2 p - (l + r)
+template <typename T>
+__device__ __forceinline__ T lap_add(T q, T l, T r, T p) {
+  if constexpr (is_df<T>::value) return dfl::df_lap_add(q, l, r, p);
+  else return q + neg_lap(l, r, p);
 }
 
 // u = p - 2 z~ (one rounding, the same as p - z at full scale)
 template <typename T>
 __device__ __forceinline__ c2_t<T> sub2(c2_t<T> p, c2_t<T> zh) {
-  if constexpr (is_df<T>::value) return mk<T>(p.x - df_scale(zh.x, 2.f), p.y - df_scale(zh.y, 2.f));
+  if constexpr (is_df<T>::value) return mk<T>(dfl::df_sub2(p.x, zh.x), dfl::df_sub2(p.y, zh.y));
   else return mk<T>(fma(T(-2), zh.x, p.x), fma(T(-2), zh.y, p.y));
 }
 
@@ -466,7 +474,7 @@ __device__ __forceinline__ void local_forward(const c2_t<T> (&p)[SEG], c2_t<T> (
       if (k <= M) v = var_forward<T, IMAG>(prev, left, p[j], right, alpha, vbf, vh, k);
     } else {
       // t = e~_{k-1} - lap_k,  lap_k = left - 2 p_k + right
-      const c2_t<T> t = mk<T>(prev.x + neg_lap(left.x, right.x, p[j].x), prev.y + neg_lap(left.y, right.y, p[j].y));
+      const c2_t<T> t = mk<T>(lap_add(prev.x, left.x, right.x, p[j].x), lap_add(prev.y, left.y, right.y, p[j].y));
       if (k <= M) v = cf_mul<T, IMAG>(alpha[k], t);
     }
     e[j] = v;
@@ -512,7 +520,7 @@ __device__ __forceinline__ void stream_forward(GetP getp, c2_t<T> (&e)[SEG], con
     if constexpr (VAR) {
       if (k <= M) v = var_forward<T, IMAG>(prev, pm, pc, pn, alpha, vbf, vh, k);
     } else {
-      const c2 t = mk<T>(prev.x + neg_lap(pm.x, pn.x, pc.x), prev.y + neg_lap(pm.y, pn.y, pc.y));
+      const c2 t = mk<T>(lap_add(prev.x, pm.x, pn.x, pc.x), lap_add(prev.y, pm.y, pn.y, pc.y));
       if (k <= M) v = cf_mul<T, IMAG>(alpha[k], t);
     }
     e[j] = v;
