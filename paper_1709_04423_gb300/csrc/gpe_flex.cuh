@@ -239,23 +239,29 @@ __device__ __forceinline__ void flex_body(const Sweep2Args<T>& A, const FlexTile
   V* cbv = reinterpret_cast<V*>(cb);
   auto slot = [&](int q) { return SPLIT ? (((q << lw) + c) << 1) + comp : (q << lw) + c; };
   auto pair_slot = [&](int q) { return SPLIT ? slot(q) ^ 1 : slot(q); };  // the other component's
-  auto get = [&](int k) -> V { return X::part(at(c, k), comp); };
+  // this segment's points in the tile (point k0 + j at seg[j], the two next to it at
+  // seg[-2] and seg[SEG + 1]) and how many of them the line has
+  c2* seg = tile + c * F.P + k0 + s;
+  const int jm = M - k0 + 1;
+  auto get = [&](int j) -> V { return X::part(seg[j], comp); };
   const V vzero = X::zero();
   V z[SEG];
+#pragma unroll
+  for (int j = 0; j < SEG; ++j) z[j] = vzero;  // (unset on one path they would stay live around a caller's loop)
   if (solving) {
-    V pm = k0 > 1 && k0 - 1 <= M ? get(k0 - 1) : vzero, pc = k0 <= M ? get(k0) : vzero, prev = vzero;
+    V pm = s > 0 && jm >= 0 ? get(-2) : vzero, pc = jm > 0 ? get(0) : vzero, prev = vzero;
 #pragma unroll
     for (int j = 0; j < SEG; ++j) {
       const int k = k0 + j;
-      const V pn = k + 1 <= M ? get(k + 1) : vzero;
+      const V pn = j + 1 < jm ? get(j + 1 < SEG ? j + 1 : SEG + 1) : vzero;
       V v = vzero;
       if constexpr (VAR) {
-        const c2 h = k <= M ? A.vh[k] : zero;
+        const c2 h = j < jm ? A.vh[k] : zero;
         const V lv = X::lapv(pm, pn, pc, h);
-        v = X::fma(k <= M ? A.alpha[k] : zero, prev, X::mul(k <= M ? A.vbf[k] : zero, lv, comp), comp);
+        v = X::fma(j < jm ? A.alpha[k] : zero, prev, X::mul(j < jm ? A.vbf[k] : zero, lv, comp), comp);
       } else {
         const V t = X::lap_add(prev, pm, pn, pc);
-        v = X::mul(k <= M ? A.alpha[k] : zero, t, comp);
+        v = X::mul(j < jm ? A.alpha[k] : zero, t, comp);
       }
       z[j] = v;
       prev = v;
@@ -264,7 +270,7 @@ __device__ __forceinline__ void flex_body(const Sweep2Args<T>& A, const FlexTile
     }
     V Bend = z[SEG - 1];
 #pragma unroll
-    for (int j = 0; j < SEG; ++j) if (k0 + j == M) Bend = z[j];
+    for (int j = 0; j < SEG; ++j) if (j + 1 == jm) Bend = z[j];
     if (s < F.nseg) cfv[slot(s)] = Bend;
   }
   __syncthreads();
@@ -287,7 +293,7 @@ __device__ __forceinline__ void flex_body(const Sweep2Args<T>& A, const FlexTile
     auto fwd = [&](auto nj) {
 #pragma unroll
       for (int j = 0; j < decltype(nj)::value; ++j)
-        if (k0 + j <= M) z[j] = X::fma_pair(__ldg(&A.gf[k0 + j]), Ein, Eo, z[j], comp);
+        if (j < jm) z[j] = X::fma_pair(__ldg(&A.gf[k0 + j]), Ein, Eo, z[j], comp);
     };
     if (SEG > 4 && A.cpts == 4) fwd(std::integral_constant<int, (SEG > 4 ? 4 : SEG)>());
     else if (SEG > 8 && A.cpts == 8) fwd(std::integral_constant<int, (SEG > 8 ? 8 : SEG)>());
@@ -296,9 +302,8 @@ __device__ __forceinline__ void flex_body(const Sweep2Args<T>& A, const FlexTile
     V next = vzero;
 #pragma unroll
     for (int j = SEG - 1; j >= 0; --j) {
-      const int k = k0 + j;
-      next = X::fma(k <= M ? bk[k] : zero, next, z[j], comp);
-      if (k > M) next = vzero;
+      next = X::fma(j < jm ? bk[k0 + j] : zero, next, z[j], comp);
+      if (j >= jm) next = vzero;
       z[j] = next;
     }
     if (s < F.nseg) cbv[slot(s)] = z[0];
@@ -325,7 +330,7 @@ __device__ __forceinline__ void flex_body(const Sweep2Args<T>& A, const FlexTile
     auto bwd = [&](auto nj) {
 #pragma unroll
       for (int j = SEG - decltype(nj)::value; j < SEG; ++j)
-        if (k0 + j <= M) z[j] = X::fma_pair(__ldg(&A.gb[k0 + j]), Zin, Zo, z[j], comp);
+        if (j < jm) z[j] = X::fma_pair(__ldg(&A.gb[k0 + j]), Zin, Zo, z[j], comp);
     };
     if (SEG > 4 && whole && A.cpts == 4) bwd(std::integral_constant<int, (SEG > 4 ? 4 : SEG)>());
     else if (SEG > 8 && whole && A.cpts == 8) bwd(std::integral_constant<int, (SEG > 8 ? 8 : SEG)>());
@@ -335,7 +340,7 @@ __device__ __forceinline__ void flex_body(const Sweep2Args<T>& A, const FlexTile
     if constexpr (AXIS0) {
 #pragma unroll
       for (int j = 0; j < SEG; ++j)
-        if (k0 + j <= M && solver) X::set(at(c, k0 + j), comp, X::sub2(get(k0 + j), z[j]));
+        if (j < jm && solver) X::set(seg[j], comp, X::sub2(get(j), z[j]));
     } else {
       const int L = L0 + c, st = (int)G.stride;
       const long base = solver ? line_base(G, L) : 0;
@@ -345,14 +350,14 @@ __device__ __forceinline__ void flex_body(const Sweep2Args<T>& A, const FlexTile
 #pragma unroll
       for (int j = 0; j < SEG; ++j) {
         const int k = k0 + j;
-        V u = k <= M ? X::sub2(get(k), z[j]) : vzero;
+        V u = j < jm ? X::sub2(get(j), z[j]) : vzero;
         if constexpr (CLOSE) {
           c2 f = X::full(u, comp);
-          if (k <= M && solver)
+          if (j < jm && solver)
             f = half_phase<T, IMAG>(A, f, base + (long)k * st, ci, G.axis == 2 ? cf2 : k, G.axis == 2 ? k : cf2);
           u = X::part(f, comp);
         }
-        if (k <= M && solver) {
+        if (j < jm && solver) {
           if (GPE_CHECK(base + (long)k * st < lim, 303)) X::set(line[(long)k * st], comp, u);
           if (LAST) tacc += A.w_axis[k] * X::sq(u);
         }

@@ -780,6 +780,7 @@ __device__ __forceinline__ void tsweep_body(const Sweep2Args<T>& A, int L0, c2_t
   pdl_release();
   constexpr bool kF64 = std::is_same<T, double>::value;
   const int per_line = (n + 31) >> 5;  // n <= 512: at most 16 chunks
+  constexpr int kLoads = sizeof(c2) == 8 ? 8 : 4;  // a lane's loads in flight
   const c2* in = A.src ? A.src : A.psi;
   const T* rin = reinterpret_cast<const T*>(in);  // RL
   const long lim = G.points();  // complex values (RL: reals) of the array
@@ -868,16 +869,16 @@ __device__ __forceinline__ void tsweep_body(const Sweep2Args<T>& A, int L0, c2_t
         c2 fline;
         T vline;
         if (!pend) line_part(L0 + c, fline, vline);
-        for (int q0 = 0; q0 < per_line; q0 += 4) {
-          c2 v[4];
+        for (int q0 = 0; q0 < per_line; q0 += kLoads) {
+          c2 v[kLoads];
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
+          for (int i = 0; i < kLoads; ++i) {
             const int k = (q0 + i) * 32 + lane;
             v[i] = (line_ok && k >= 1 && k <= M && GPE_CHECK((long)gbase + k < lim, 214)) ? in[gbase + k]
                                                                                           : mk<T>(0, 0);
           }
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
+          for (int i = 0; i < kLoads; ++i) {
             const int k = (q0 + i) * 32 + lane;
             if (k >= n) break;
             c2 w = v[i];
