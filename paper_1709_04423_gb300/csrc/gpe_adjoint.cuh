@@ -32,13 +32,36 @@ struct AdjPhaseArgs {
   double* dJdg;        // FP64 accumulator (device scalar); the last block adds this step's sum
 };
 
+// The adjoint of N at one point: the updated lambda, with dt s added to dV and
+// dt s |p|^2 to gacc.
+template <typename T>
+__device__ __forceinline__ c2_t<T> adjoint_phase_point(c2_t<T> p, c2_t<T> l, T V, T dt, T g, double& dV, T& gacc) {
+  const T dens = p.x * p.x + p.y * p.y;
+  const T th = dt * (V + g * dens);
+  // rotations with the forward's coefficients (rot_coefs): cos th = 1 + cm1
+  T sn, cm1;
+  rot_coefs<T>(th, sn, cm1);
+  const c2_t<T> u = rot_apply<T>(p, sn, cm1);  // exp(-i th) p
+  const T s = l.x * u.y - l.y * u.x;           // Im(conj(lam) u)
+  const T ds = dt * s;
+  dV += (double)ds;
+  gacc += ds * dens;
+  const T c2g = T(2) * g * ds;
+  // exp(i th) lam + 2 g dt s p
+  return mk<T>((l.x + fma(cm1, l.x, -(sn * l.y))) + c2g * p.x, (l.y + fma(cm1, l.y, sn * l.x)) + c2g * p.y);
+}
+
+// As a pass of its own, after x sweeps that do not apply it themselves
+// (tsweep_body with ADJ does).
 template <typename T>
 __global__ void __launch_bounds__(256) adjoint_phase_kernel(AdjPhaseArgs<T> A) {
   __shared__ double red_smem[32];
   T gacc = T(0);
+  pdl_wait();
+  pdl_release();
   for (long q = (long)blockIdx.x * blockDim.x + threadIdx.x; q < A.np; q += (long)gridDim.x * blockDim.x) {
     const c2_t<T> p = A.phi[q];
-    c2_t<T> l = A.lam[q];
+    const c2_t<T> l = A.lam[q];
     T Vq;
     if (A.V) {
       Vq = A.V[q];
@@ -47,20 +70,9 @@ __global__ void __launch_bounds__(256) adjoint_phase_kernel(AdjPhaseArgs<T> A) {
       const long r = q / A.nx;
       Vq = A.vx[i] + A.vy[(int)(r % A.ny)] + A.vz[(int)(r / A.ny)];
     }
-    const T dens = p.x * p.x + p.y * p.y;
-    const T th = A.dt * (Vq + A.g * dens);
-    // rotations with the forward's coefficients (rot_coefs): cos th = 1 + cm1
-    T sn, cm1;
-    rot_coefs<T>(th, sn, cm1);
-    const c2_t<T> u = rot_neg<T>(p, th);                                // exp(-i th) p
-    const T s = l.x * u.y - l.y * u.x;                                  // Im(conj(lam) u)
-    const T ds = A.dt * s;
-    A.dJdV[q] += (double)ds;
-    gacc += ds * dens;
-    const T c2g = T(2) * A.g * ds;
-    // exp(i th) lam + 2 g dt s p
-    l = mk<T>((l.x + fma(cm1, l.x, -(sn * l.y))) + c2g * p.x, (l.y + fma(cm1, l.y, sn * l.x)) + c2g * p.y);
-    A.lam[q] = l;
+    double dV = A.dJdV[q];
+    A.lam[q] = adjoint_phase_point<T>(p, l, Vq, A.dt, A.g, dV, gacc);
+    A.dJdV[q] = dV;
   }
   double v[1] = {(double)gacc}, tot[1];  // FP64 from the per-thread sums on
   block_sum<1>(v, red_smem);

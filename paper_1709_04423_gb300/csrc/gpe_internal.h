@@ -177,6 +177,7 @@ struct gp_handle {
   long adj_ckpt_cap = 0;      // states the buffer holds
   void* adj_traj = nullptr;   // K states
   long adj_traj_cap = 0;
+  long adj_traj_seg = -1;     // the segment whose states the buffer holds (-1: none)
   void* adj_lam = nullptr;    // one state
   double* adj_dJdV = nullptr; // npoints doubles
   double* adj_dJdg = nullptr; // one double

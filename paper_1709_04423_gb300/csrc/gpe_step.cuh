@@ -130,26 +130,26 @@ inline bool xy_fused(const gp_handle* h) {
 
 // ---- shared-memory tile x sweep
 // (RL: a.geom.nlines real lines, two per tile column; VAR: a rho axis)
-template <typename T, bool IMAG, bool FIRST, bool LAST, int SEG, bool RL = false, bool VAR = false>
+template <typename T, bool IMAG, bool FIRST, bool LAST, int SEG, bool RL = false, bool VAR = false, bool ADJ = false>
 unsigned launch_t(const Sweep2Args<T>& a, cudaStream_t s, bool pdl) {
   const int M = a.geom.n - 2;
   const int nseg = (M + SEG - 1) / SEG;
   const long ncols = RL ? (a.geom.nlines + 1) / 2 : a.geom.nlines;
   const unsigned blocks = (unsigned)((ncols + 31) / 32);
   const size_t smem = (size_t)a.geom.n * (kTilePitch + 3) * sizeof(c2_t<T>) + 512 * sizeof(c2_t<T>);
-  opt_in_smem((const void*)tsweep_kernel<T, IMAG, FIRST, LAST, SEG, RL, VAR>, 200 * 1024);
-  launch_k(pdl, tsweep_kernel<T, IMAG, FIRST, LAST, SEG, RL, VAR>, dim3(blocks), dim3(32 * nseg), smem, s, a);
+  opt_in_smem((const void*)tsweep_kernel<T, IMAG, FIRST, LAST, SEG, RL, VAR, ADJ>, 200 * 1024);
+  launch_k(pdl, tsweep_kernel<T, IMAG, FIRST, LAST, SEG, RL, VAR, ADJ>, dim3(blocks), dim3(32 * nseg), smem, s, a);
   count_launch();
   return blocks;
 }
 
-template <typename T, bool IMAG, bool FIRST, bool LAST, bool RL = false, bool VAR = false>
+template <typename T, bool IMAG, bool FIRST, bool LAST, bool RL = false, bool VAR = false, bool ADJ = false>
 unsigned launch_t_seg(int seg, const Sweep2Args<T>& a, cudaStream_t s, bool pdl) {
   switch (seg) {
-    case 4: return launch_t<T, IMAG, FIRST, LAST, 4, RL, VAR>(a, s, pdl);
-    case 8: return launch_t<T, IMAG, FIRST, LAST, 8, RL, VAR>(a, s, pdl);
-    case 16: return launch_t<T, IMAG, FIRST, LAST, 16, RL, VAR>(a, s, pdl);
-    default: return launch_t<T, IMAG, FIRST, LAST, 32, RL, VAR>(a, s, pdl);
+    case 4: return launch_t<T, IMAG, FIRST, LAST, 4, RL, VAR, ADJ>(a, s, pdl);
+    case 8: return launch_t<T, IMAG, FIRST, LAST, 8, RL, VAR, ADJ>(a, s, pdl);
+    case 16: return launch_t<T, IMAG, FIRST, LAST, 16, RL, VAR, ADJ>(a, s, pdl);
+    default: return launch_t<T, IMAG, FIRST, LAST, 32, RL, VAR, ADJ>(a, s, pdl);
   }
 }
 
@@ -721,6 +721,15 @@ void enqueue_finish_imag(gp_handle* h, long nsteps) {
   count_launch();
 }
 
+// Consecutive kernels overlap their launch and prologue inside this scope (FP32
+// and double-float; the FP64 form, bound by its FP64 pipe, was measured 10 %
+// slower with it).
+struct PdlScope {
+  gp_handle* h;
+  explicit PdlScope(gp_handle* hh) : h(hh) { h->pdl_now = pdl_enabled() && h->prec != GP_F64; }
+  ~PdlScope() { h->pdl_now = false; }
+};
+
 // Step 0 eagerly (imaginary time: it has no pending factor; real-time Strang:
 // it opens with N(dt/2)), then blocks of kGraphSteps steps replayed from one
 // captured graph (a block starts at an odd step in imaginary time, so its
@@ -730,14 +739,7 @@ int run_steps_t(gp_handle* h, bool imag, long nsteps) {
   if (nsteps == 0) return GP_OK;
   int rc = join_in(h);
   if (rc) return rc;
-  // consecutive sweeps overlap their launch and prologue (FP32 and
-  // double-float; the FP64 form, bound by its FP64 pipe, was measured 10 %
-  // slower with it)
-  struct PdlScope {
-    gp_handle* h;
-    explicit PdlScope(gp_handle* hh) : h(hh) { h->pdl_now = pdl_enabled() && h->prec != GP_F64; }
-    ~PdlScope() { h->pdl_now = false; }
-  } pdl_scope(h);
+  PdlScope pdl_scope(h);
   // real-time Strang: the halves between steps merged (StepForm)
   const bool merged = h->strang && !imag;
   const StepForm first_f{true, !merged}, next_f{!merged, !merged};
@@ -812,11 +814,7 @@ int time_sweeps_graph_t(gp_handle* h, bool imag, int reps, double* ms_out) {
   int rc = join_in(h);
   if (rc) return rc;
   for (int d = 0; d < 3; ++d) ms_out[d] = 0.0;
-  struct PdlScope {
-    gp_handle* h;
-    explicit PdlScope(gp_handle* hh) : h(hh) { h->pdl_now = pdl_enabled() && h->prec != GP_F64; }
-    ~PdlScope() { h->pdl_now = false; }
-  } pdl_scope(h);
+  PdlScope pdl_scope(h);
   for (long t = 0; t < 2; ++t) enqueue_step<T>(h, imag, slots_of_step(imag, t));
   NormSlots ns;
   if (imag) {
@@ -906,9 +904,10 @@ int run_observables_t(gp_handle* h, double* dens_dev, double* sums_out = nullptr
 
 // ---------------------------------------------------------------- adjoint
 // Sweep of the adjoint state along axis d with the dt -> -dt coefficients
-// (the conjugate-transposed Crank-Nicolson map).
+// (the conjugate-transposed Crank-Nicolson map).  The tile x sweep also applies
+// the adjoint of N at the step's input phi; returns whether it did.
 template <typename T>
-void enqueue_adj_sweep(gp_handle* h, int d) {
+bool enqueue_adj_sweep(gp_handle* h, int d, const void* phi) {
   Sweep2Args<T> a;
   std::memset(&a, 0, sizeof(a));
   a.psi = (c2_t<T>*)h->adj_lam;
@@ -922,10 +921,25 @@ void enqueue_adj_sweep(gp_handle* h, int d) {
   a.cdepth = h->cdepth[MODE_REAL_ADJ][d][si];
   a.cpts = h->cpts[MODE_REAL_ADJ][d][si];
   if (d == 0 && h->tile_x && h->pipe_x) launch_p_seg<T, false, false, false, true>(seg, a, h->work, h->pdl_now);
-  else if (d == 0 && h->tile_x) launch_t_seg<T, false, false, false>(seg, a, h->work, h->pdl_now);
+  else if (d == 0 && h->tile_x) {
+    a.adj_phi = (const c2_t<T>*)phi;
+    a.adj_dJdV = h->adj_dJdV;
+    a.adj_partials = h->partials;
+    a.adj_counter = h->counter;
+    a.adj_dJdg = h->adj_dJdg;
+    a.V = (const T*)h->Vt;
+    a.vx = (const T*)h->vt[0];
+    a.vy = (const T*)h->vt[1];
+    a.vz = (const T*)h->vt[2];
+    a.dt = (T)h->adj_dt;
+    a.g = (T)h->adj_g;
+    launch_t_seg<T, false, false, false, false, false, true>(seg, a, h->work, h->pdl_now);
+    return true;
+  }
   else if (d == 0) launch_x_seg<T, false, false, false>(seg, a, h->work, h->pdl_now);
   else if (h->pipe_c) launch_p_seg<T, false, false, false, false>(seg, a, h->work, h->pdl_now);
   else launch_c_seg<T, false, false>(seg, h->keep_c, a, h->work, h->pdl_now);
+  return false;
 }
 
 template <typename T>
@@ -948,22 +962,48 @@ void enqueue_adj_phase(gp_handle* h, const void* phi) {
   a.counter = h->counter;
   a.dJdg = h->adj_dJdg;
   const int blocks = (int)std::min<long>((h->np + 255) / 256, 152L * 16);
-  adjoint_phase_kernel<T><<<blocks, 256, 0, h->work>>>(a);
+  launch_k(h->pdl_now, adjoint_phase_kernel<T>, dim3(blocks), dim3(256), 0, h->work, a);
   count_launch();
+}
+
+// len steps from the state in psi whose inputs go to the trajectory buffer:
+// step j reads entry j and writes entry j + 1, the last one psi.
+template <typename T>
+void enqueue_recorded(gp_handle* h, int len, bool to_psi) {
+  const size_t sbytes = (size_t)h->np * h->esize;
+  char* traj = (char*)h->adj_traj;
+  void* const psi = h->psi;
+  for (int j = 0; j < len; ++j) {
+    if (j + 1 == len && !to_psi) break;
+    h->psi = j + 1 == len ? psi : traj + (size_t)(j + 1) * sbytes;
+    enqueue_step<T>(h, false, NormSlots{}, nullptr, traj + (size_t)j * sbytes);
+  }
+  h->psi = psi;
 }
 
 // Forward run of nsteps real-time steps from the current state, keeping the
 // state at steps 0, K, 2K, ... (buffers sized by the caller of this function).
+// The last segment's steps go straight into the trajectory buffer, where the
+// reverse pass, which starts with them, finds them without recomputing.
 template <typename T>
 int adjoint_forward_t(gp_handle* h, long nsteps, int K) {
   const long nck = (nsteps + K - 1) / K;
+  const size_t sbytes = (size_t)h->np * h->esize;
+  h->adj_traj_seg = -1;
   for (long c = 0; c < nck; ++c) {
     int rc = join_in(h);
     if (rc) return rc;
-    GP_CUDA(cudaMemcpyAsync((char*)h->adj_ckpt + (size_t)c * h->np * h->esize, h->psi, (size_t)h->np * h->esize,
-                            cudaMemcpyDeviceToDevice, h->work));
+    GP_CUDA(cudaMemcpyAsync((char*)h->adj_ckpt + (size_t)c * sbytes, h->psi, sbytes, cudaMemcpyDeviceToDevice,
+                            h->work));
+    if (c == nck - 1) {
+      PdlScope pdl(h);
+      GP_CUDA(cudaMemcpyAsync(h->adj_traj, h->psi, sbytes, cudaMemcpyDeviceToDevice, h->work));
+      enqueue_recorded<T>(h, (int)(nsteps - c * K), true);
+      GP_CUDA(cudaGetLastError());
+      h->adj_traj_seg = c;
+    }
     if ((rc = join_out(h))) return rc;
-    if ((rc = run_steps_t<T>(h, false, std::min<long>(K, nsteps - c * K)))) return rc;
+    if (c < nck - 1 && (rc = run_steps_t<T>(h, false, K))) return rc;
   }
   return GP_OK;
 }
@@ -984,25 +1024,26 @@ int adjoint_backward_t(gp_handle* h, double* dJdV_dev, void* lam0_dev) {
   if (rc) return rc;
   GP_CUDA(cudaMemsetAsync(h->adj_dJdV, 0, (size_t)h->np * sizeof(double), h->work));
   GP_CUDA(cudaMemsetAsync(h->adj_dJdg, 0, sizeof(double), h->work));
-  void* psi_saved = h->psi;
   const double g_now = h->g, dt_now = h->dt;
+  PdlScope pdl(h);
   h->g = h->adj_g;  // the forward's g and dt drive the recomputation
   h->dt = h->adj_dt;
   for (long c = nck - 1; c >= 0; --c) {
     const long t0 = c * K;
     const int len = (int)std::min<long>(K, nsteps - t0);
     char* traj = (char*)h->adj_traj;
-    cudaMemcpyAsync(traj, (const char*)h->adj_ckpt + (size_t)c * sbytes, sbytes, cudaMemcpyDeviceToDevice, h->work);
-    for (int j = 0; j + 1 < len; ++j) {
-      h->psi = traj + (size_t)(j + 1) * sbytes;
-      enqueue_step<T>(h, false, NormSlots{}, nullptr, traj + (size_t)j * sbytes);
+    if (h->adj_traj_seg != c) {
+      cudaMemcpyAsync(traj, (const char*)h->adj_ckpt + (size_t)c * sbytes, sbytes, cudaMemcpyDeviceToDevice, h->work);
+      enqueue_recorded<T>(h, len, false);
+      h->adj_traj_seg = c;
     }
     for (int j = len - 1; j >= 0; --j) {
-      for (int d = h->dim - 1; d >= 0; --d) enqueue_adj_sweep<T>(h, d);
-      enqueue_adj_phase<T>(h, traj + (size_t)j * sbytes);
+      const char* phi = traj + (size_t)j * sbytes;
+      bool done = false;
+      for (int d = h->dim - 1; d >= 0; --d) done = enqueue_adj_sweep<T>(h, d, phi);
+      if (!done) enqueue_adj_phase<T>(h, phi);
     }
   }
-  h->psi = psi_saved;
   h->g = g_now;
   h->dt = dt_now;
   h->adj_dJdV = dJdV_keep;

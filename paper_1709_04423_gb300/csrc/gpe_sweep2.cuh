@@ -52,6 +52,7 @@
 #pragma once
 #include <type_traits>
 
+#include "gpe_adjoint.cuh"
 #include "gpe_common.cuh"
 
 namespace gpe {
@@ -114,6 +115,13 @@ struct Sweep2Args {
   // cdepth segments and reach the first (last) cpts points of a segment, cpts
   // one of 4, 8, 12; 0 = every segment and point
   int cdepth, cpts;
+  // the reverse step's x sweep (ADJ): the adjoint of N after it, at the step's
+  // input adj_phi (V, dt, g above), with the gradients' accumulators
+  const c2_t<T>* adj_phi;
+  double* adj_dJdV;
+  double* adj_partials;
+  unsigned int* adj_counter;
+  double* adj_dJdg;
 };
 
 // Sub-step N at one point in factor form: p <- F exp(-i a) p (real time) or F exp(-a) p
@@ -763,7 +771,11 @@ constexpr int kTilePitch = 33;
 // density and potential, and with real coefficients the complex solve of a
 // column is the two real solves.
 // VAR: the rho axis of an axial trap (see Sweep2Args::vab).
-template <typename T, bool IMAG, bool FIRST, bool LAST, int SEG, bool RL = false, bool VAR = false>
+// ADJ: a reverse step's x sweep, which applies the adjoint of N (adjoint_phase_point)
+// to its output on the way out: one pass over lambda less than with a kernel of
+// its own.  (With programmatic launches in the reverse pass and the last segment
+// kept from the forward run: 96^3 FP32, 50 steps forward and back, 4.50 -> 2.72 ms.)
+template <typename T, bool IMAG, bool FIRST, bool LAST, int SEG, bool RL = false, bool VAR = false, bool ADJ = false>
 __device__ __forceinline__ void tsweep_body(const Sweep2Args<T>& A, int L0, c2_t<T>* sc, c2_t<T> (*cf)[33],
                                             c2_t<T> (*cb)[33], double* red_smem) {
   static_assert(!(RL && (LAST || is_df<T>::value || !IMAG)), "packed real lines: imaginary-time x sweeps of 2d/3d");
@@ -943,6 +955,7 @@ __device__ __forceinline__ void tsweep_body(const Sweep2Args<T>& A, int L0, c2_t
   }
   __syncthreads();
   // ---- store (tile end points are zero)
+  [[maybe_unused]] T gacc = T(0);  // ADJ
   for (int c = s; c < nl; c += nwarps) {
     if constexpr (RL) {
       T* rout = reinterpret_cast<T*>(A.psi);
@@ -954,20 +967,52 @@ __device__ __forceinline__ void tsweep_body(const Sweep2Args<T>& A, int L0, c2_t
           if (GPE_CHECK((long)Lb * G.nx + k < lim, 217)) rout[Lb * G.nx + k] = tile[k * kTilePitch + c].y;
     } else {
       const int gbase = (L0 + c) * G.nx;
-      for (int k = lane; k < n; k += 32)
-        if (GPE_CHECK((long)gbase + k < lim, 218)) A.psi[gbase + k] = tile[k * kTilePitch + c];
+      if constexpr (ADJ) {
+        // (end points: lambda is zero there, so nothing changes)
+        const T vline = A.V ? T(0) : A.vy[(L0 + c) % G.ny] + A.vz[(L0 + c) / G.ny];
+        for (int q0 = 0; q0 < per_line; q0 += 4) {
+          c2 p[4];
+          double dV[4];
+          T V[4];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const int k = (q0 + i) * 32 + lane;
+            const bool ok = k < n && GPE_CHECK((long)gbase + k < lim, 219);
+            p[i] = ok ? A.adj_phi[gbase + k] : mk<T>(0, 0);
+            dV[i] = ok ? A.adj_dJdV[gbase + k] : 0.0;
+            V[i] = ok ? (A.V ? A.V[gbase + k] : A.vx[k] + vline) : T(0);
+          }
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const int k = (q0 + i) * 32 + lane;
+            if (k < n && GPE_CHECK((long)gbase + k < lim, 219)) {
+              A.psi[gbase + k] = adjoint_phase_point<T>(p[i], tile[k * kTilePitch + c], V[i], A.dt, A.g, dV[i], gacc);
+              A.adj_dJdV[gbase + k] = dV[i];
+            }
+          }
+        }
+      } else {
+        for (int k = lane; k < n; k += 32)
+          if (GPE_CHECK((long)gbase + k < lim, 218)) A.psi[gbase + k] = tile[k * kTilePitch + c];
+      }
     }
+  }
+  if constexpr (ADJ) {
+    double v[1] = {(double)gacc}, tot[1];  // FP64 from the per-thread sums on
+    __syncthreads();                       // red_smem is free
+    block_sum<1>(v, red_smem);
+    if (grid_sum_last<1>(v, A.adj_partials, A.adj_counter, tot, red_smem) && threadIdx.x == 0) *A.adj_dJdg += tot[0];
   }
   finish_norm<T, LAST>(nval, A.parts_out);
 }
 
-template <typename T, bool IMAG, bool FIRST, bool LAST, int SEG, bool RL = false, bool VAR = false>
+template <typename T, bool IMAG, bool FIRST, bool LAST, int SEG, bool RL = false, bool VAR = false, bool ADJ = false>
 __global__ void __launch_bounds__(512) tsweep_kernel(Sweep2Args<T> A) {
   extern __shared__ __align__(16) unsigned char tsmem_raw[];
   __shared__ c2_t<T> cf[16][33], cb[16][33];
   __shared__ double red_smem[32];
-  tsweep_body<T, IMAG, FIRST, LAST, SEG, RL, VAR>(A, blockIdx.x * 32, reinterpret_cast<c2_t<T>*>(tsmem_raw), cf, cb,
-                                         red_smem);
+  tsweep_body<T, IMAG, FIRST, LAST, SEG, RL, VAR, ADJ>(A, blockIdx.x * 32, reinterpret_cast<c2_t<T>*>(tsmem_raw), cf, cb,
+                                                       red_smem);
 }
 
 // ---------------------------------------------------------------- fused x + y sweeps (3d, FP32)
