@@ -426,9 +426,15 @@ bool tma_x_fits(const gp_handle* h, int seg) {
 }
 
 int read_dev_err(gp_handle* h, const char* who) {
-  int e = 0;
-  GP_CUDA(cudaMemcpyAsync(&e, h->dev_err, sizeof(int), cudaMemcpyDeviceToHost, h->work));
+  GP_CUDA(cudaMemcpyAsync(h->obs_host + 8, h->dev_err, sizeof(int), cudaMemcpyDeviceToHost, h->work));
   GP_CUDA(cudaStreamSynchronize(h->work));
+  return take_dev_err(h, who);
+}
+
+// The device error flag that a transfer has brought to obs_host[8].
+int take_dev_err(gp_handle* h, const char* who) {
+  int e = 0;
+  std::memcpy(&e, h->obs_host + 8, sizeof(int));
   if (e == 0) return GP_OK;
   GP_CUDA(cudaMemsetAsync(h->dev_err, 0, sizeof(int), h->work));
   GP_CUDA(cudaStreamSynchronize(h->work));
@@ -678,7 +684,7 @@ int init_handle(gp_handle** out, int geom, int dim, const int n[3], const double
     if (e != cudaSuccess) return bail(fail(GP_ERR_CUDA, std::string("cudaStreamCreate: ") + cudaGetErrorString(e)));
     e = cudaEventCreateWithFlags(&h->ev_in, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_out, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaMallocHost((void**)&h->obs_host, 8 * sizeof(double));
+    if (e == cudaSuccess) e = cudaMallocHost((void**)&h->obs_host, 9 * sizeof(double));
     if (e != cudaSuccess) return bail(fail(GP_ERR_CUDA, std::string("gp_init: ") + cudaGetErrorString(e)));
   }
   const size_t tsz = prec == GP_F64 ? sizeof(double) : prec == GP_DF64 ? sizeof(df64) : sizeof(float);
@@ -781,7 +787,6 @@ int init_handle(gp_handle** out, int geom, int dim, const int n[3], const double
   for (int d = 0; d < dim; ++d) maxblocks = std::max(maxblocks, h->np / h->n[d] / 4 + 1);
   if ((rc = dev_alloc(h, (void**)&h->partials, (size_t)maxblocks * 8 * sizeof(double)))) return bail(rc);
   if ((rc = dev_alloc(h, (void**)&h->counter, 64))) return bail(rc);
-  if ((rc = dev_alloc(h, (void**)&h->dev_err, 64))) return bail(rc);
   h->tma_limit_ns = (unsigned long long)env_int("GPE_WAIT_LIMIT_MS", 1000) * 1000000ull;
   {
     // one norm sum per block of any last sweep: 32 lines per block (tiles and
@@ -792,7 +797,9 @@ int init_handle(gp_handle** out, int geom, int dim, const int n[3], const double
     for (int i = 0; i < 2; ++i)
       if ((rc = dev_alloc(h, (void**)&h->parts[i], (size_t)maxparts * sizeof(double)))) return bail(rc);
   }
-  if ((rc = dev_alloc(h, (void**)&h->obs_out, 8 * sizeof(double)))) return bail(rc);
+  // the observables' sums and, after them, the error flag: one transfer brings both
+  if ((rc = dev_alloc(h, (void**)&h->obs_out, 9 * sizeof(double)))) return bail(rc);
+  h->dev_err = reinterpret_cast<int*>(h->obs_out + 8);
   {
     cudaError_t e = cudaStreamSynchronize(h->work);
     if (e != cudaSuccess) return bail(fail(GP_ERR_CUDA, std::string("gp_init: ") + cudaGetErrorString(e)));
@@ -1406,13 +1413,12 @@ int gp_observables(gp_handle* h, gp_obs* out, double* density, int density_on_de
   }
   rc = run_observables_any(h, ddev);
   if (rc) return rc;
-  if ((rc = read_dev_err(h, "gp_observables"))) return rc;
-  GP_CUDA(cudaMemcpyAsync(h->obs_host, h->obs_out, 7 * sizeof(double), cudaMemcpyDeviceToHost, h->work));
+  GP_CUDA(cudaMemcpyAsync(h->obs_host, h->obs_out, 9 * sizeof(double), cudaMemcpyDeviceToHost, h->work));
   if (density && !density_on_device)
     GP_CUDA(cudaMemcpyAsync(density, ddev, (size_t)h->np * sizeof(double), cudaMemcpyDeviceToHost, h->work));
   GP_CUDA(cudaStreamSynchronize(h->work));
-  rc = join_out(h);
-  if (rc) return rc;
+  if ((rc = take_dev_err(h, "gp_observables"))) return rc;
+  // (the work is done: nothing for the caller's stream to wait for)
   const double* S = h->obs_host;
   const double N = S[0];
   out->norm = N;

@@ -163,8 +163,8 @@ struct gp_handle {
   size_t series_cap = 0;  // launch the sweeps as programmatic dependents (inside gp_step_*)
   double* partials = nullptr;
   unsigned int* counter = nullptr;
-  double* obs_out = nullptr;  // [8]
-  double* obs_host = nullptr; // pinned [8]
+  double* obs_out = nullptr;  // [8], then the error flag
+  double* obs_host = nullptr; // pinned [9]
   double* dens_scratch = nullptr;
   cudaGraphExec_t graph[2] = {nullptr, nullptr};
   // adjoint: checkpoints of the last gp_adjoint_forward and scratch
@@ -218,6 +218,7 @@ int tile_seg(int M);
 bool plane_fits(const gp_handle* h, int seg);  // the fused x + y sweep kernel takes this grid and segment length
 bool tma_fits(const gp_handle* h, int seg);    // the TMA y/z sweeps take this grid and segment length
 bool tma_x_fits(const gp_handle* h, int seg);  // the TMA x sweep takes this grid and segment length
+int take_dev_err(gp_handle* h, const char* who);
 int read_dev_err(gp_handle* h, const char* who);  // GP_ERR_TIMEOUT (and clears it) if a device wait gave up
 
 int dev_alloc(gp_handle* h, void** p, size_t bytes);
