@@ -757,6 +757,24 @@ __global__ void __launch_bounds__(512) colsweep_kernel(Sweep2Args<T> A) {
                                                      cb, red_smem);
 }
 
+// ---------------------------------------------------------------- asynchronous copies
+__device__ __forceinline__ unsigned smem_u32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
+
+// async copy of one complex value (8 or 16 bytes); src_bytes = 0 zero-fills
+template <typename T>
+__device__ __forceinline__ void cp_async_c2(c2_t<T>* dst, const c2_t<T>* src, bool valid) {
+  const unsigned d = smem_u32(dst);
+  if constexpr (sizeof(c2_t<T>) == 16) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(d), "l"(src), "r"(valid ? 16 : 0));
+  } else {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(d), "l"(src), "r"(valid ? 8 : 0));
+  }
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::); }
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N)); }
+
 // ---------------------------------------------------------------- x sweep (2d/3d)
 // Tile of 32 x lines in shared memory, transposed ([point][line], pitch 33).
 // blockDim.x >= 32 * nseg (<= 512); dynamic shared memory: coefficients
@@ -793,6 +811,7 @@ __device__ __forceinline__ void tsweep_body(const Sweep2Args<T>& A, int L0, c2_t
   constexpr bool kF64 = std::is_same<T, double>::value;
   const int per_line = (n + 31) >> 5;  // n <= 512: at most 16 chunks
   constexpr int kLoads = sizeof(c2) == 8 ? 8 : 4;  // a lane's loads in flight
+  constexpr bool kAsync = sizeof(c2) == 8;
   const c2* in = A.src ? A.src : A.psi;
   const T* rin = reinterpret_cast<const T*>(in);  // RL
   const long lim = G.points();  // complex values (RL: reals) of the array
@@ -843,6 +862,8 @@ __device__ __forceinline__ void tsweep_body(const Sweep2Args<T>& A, int L0, c2_t
     if (lane == 0) red_smem[0] = f;
   }
   const int w0 = (pend && nwarps > 1) ? 1 : 0;  // first loading warp
+  // (lines of a few chunks have no more loads to put in flight: 64^3 5.0 -> 5.2 us)
+  const bool async = kAsync && !RL && pend && n > 96;
   if (s >= w0) {
     for (int c = s - w0; c < 32; c += nwarps - w0) {
       const bool line_ok = c < nl;
@@ -878,6 +899,16 @@ __device__ __forceinline__ void tsweep_body(const Sweep2Args<T>& A, int L0, c2_t
         }
       } else {
         const int gbase = (L0 + c) * G.nx;
+        // a pending factor, FP32: raw, straight into the tile, every copy of the
+        // block in flight at once (120 x 101 x 90 x sweep 13.6 -> 11.2 us; FP64 and
+        // double-float tiles of 16-byte points lost 2 and 6 % to it)
+        if (async) {
+          for (int k = lane; k < n; k += 32) {
+            const bool ok = line_ok && k >= 1 && k <= M && GPE_CHECK((long)gbase + k < lim, 214);
+            cp_async_c2<T>(&tile[k * kTilePitch + c], ok ? in + gbase + k : in, ok);
+          }
+          continue;
+        }
         c2 fline;
         T vline;
         if (!pend) line_part(L0 + c, fline, vline);
@@ -902,6 +933,7 @@ __device__ __forceinline__ void tsweep_body(const Sweep2Args<T>& A, int L0, c2_t
     }
   }
   if (pend) {
+    if (async) cp_async_wait_all();
     __syncthreads();
     const T scl = (T)red_smem[0];
     for (int c = s; c < nl; c += nwarps) {
@@ -1069,7 +1101,16 @@ __global__ void __launch_bounds__(1024) xyplane_kernel(Sweep2Args<float> Ax, Swe
   const int per_row = (nx + 31) >> 5;
   if (warp >= w0) {
     for (int j = warp - w0; j < ny; j += nwarps - w0) {
-      const T vline = pend ? T(0) : row_v(j);
+      // a pending factor: raw, straight into the plane, every copy of the block in
+      // flight at once (128^3: 19.3 -> 18.4 us)
+      if (pend) {
+        for (int i = lane; i < nx; i += 32) {
+          const bool ok = i >= 1 && i <= Mx && GPE_CHECK((long)j * nx + i < lim && j < ny && i < PX, 221);
+          cp_async_c2<T>(&P[j * PX + i], ok ? in + (long)j * nx + i : in, ok);
+        }
+        continue;
+      }
+      const T vline = row_v(j);
       for (int q0 = 0; q0 < per_row; q0 += 4) {
         c2 v[4];
 #pragma unroll
@@ -1082,12 +1123,13 @@ __global__ void __launch_bounds__(1024) xyplane_kernel(Sweep2Args<float> Ax, Swe
           const int i = (q0 + t) * 32 + lane;
           if (i >= nx) break;
           if (GPE_CHECK(j < ny && i < PX, 222))
-            P[j * PX + i] = (!pend && i >= 1 && i <= Mx) ? apply(v[t], j, i, vline, T(1)) : v[t];
+            P[j * PX + i] = (i >= 1 && i <= Mx) ? apply(v[t], j, i, vline, T(1)) : v[t];
         }
       }
     }
   }
   if (pend) {
+    cp_async_wait_all();
     __syncthreads();
     const T scl = (T)red_smem[0];
     for (int j = warp; j < ny; j += nwarps) {
@@ -1300,22 +1342,6 @@ namespace gpe {
 // x lines [line][point] with pitch n + 1 -- both conflict-free for the
 // lane = line reads of the solve.  The coefficient tables are loaded once per
 // block, the norm (LAST) is reduced once per block.  blockDim.x = 32 * nseg.
-
-__device__ __forceinline__ unsigned smem_u32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
-
-// async copy of one complex value (8 or 16 bytes); src_bytes = 0 zero-fills
-template <typename T>
-__device__ __forceinline__ void cp_async_c2(c2_t<T>* dst, const c2_t<T>* src, bool valid) {
-  const unsigned d = smem_u32(dst);
-  if constexpr (sizeof(c2_t<T>) == 16) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(d), "l"(src), "r"(valid ? 16 : 0));
-  } else {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(d), "l"(src), "r"(valid ? 8 : 0));
-  }
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N)); }
 
 // Issues the copies of tile `tile` into stage buffer `buf` (every thread its share).
 template <typename T, bool AXIS0>
