@@ -450,6 +450,39 @@ int tile_seg(int M) {
 
 namespace {
 
+// Defaults of 3d Cartesian grids, where the autotuner's picks agree over many
+// sizes (us per sweep of the x, y, z sweeps, the general rule's shape -> this one):
+//  * FP64 is bound by its FP64 pipe: longer segments carry less (128^3 real
+//    time 218 / 116 / 116 -> 196 / 92 / 92, 96^3 83 / 44 / 44 -> 76 / 38 / 38),
+//    unless a short axis leaves them partly empty (z of 90 points in segments of
+//    16: 53 -> 65);
+//  * FP32 states that do not stay in L2 between sweeps stream through the TMA
+//    sweeps (256^3 real 92 / 70 / 73 -> 59 / 48 / 49, 160 x 144 x 150 imaginary
+//    24 / 16 / 18 -> 18 / 11 / 15); those that do and whose xy planes nearly fill
+//    the SMs take the fused x + y sweep (128^3 imaginary 16.1 + 7.8 -> 18.4).
+void choose_shapes_3d(gp_handle* h) {
+  const int M0 = h->n[0] - 2, Ms = std::min(h->n[1], h->n[2]) - 2;
+  if (h->prec == GP_F64) {
+    if (h->tile_x && M0 > 62 && M0 <= 256) h->seg_x = 16;
+    if (h->seg_c > 0 && Ms > 90) h->seg_c = std::max(h->seg_c, Ms > 100 ? 32 : 16);
+  } else if (h->prec == GP_F32) {
+    const long bytes = h->np * (long)h->esize;
+    if (bytes > 24L << 20) {
+      if (h->tile_x && tma_x_fits(h, 16)) {
+        h->seg_x = 16;
+        h->tma_x = true;
+      }
+      if (tma_fits(h, 16)) {
+        h->seg_c = 16;
+        h->tma_c = true;
+      }
+    } else if (h->tile_x && h->n[2] >= 120 && h->n[2] <= 152 && bytes > 8L << 20 && plane_fits(h, 16)) {
+      h->seg_x = 16;
+      h->xyfuse = true;
+    }
+  }
+}
+
 void choose_shapes(gp_handle* h) {
   const int M0 = h->n[0] - 2;
   // the x tile needs (36 n + 512) complex values of shared memory (<= 200 KB)
@@ -482,6 +515,10 @@ void choose_shapes(gp_handle* h) {
   h->pipe_x = pipe && h->tile_x && h->geom != 2 && pipe_fits(h, h->n[0], true);  // (no rho-axis pipelined sweep)
   h->xyfuse = env_int("GPE_FUSE_XY", 0) != 0 && plane_fits(h, sx);
   h->pipe_c = pipe && h->dim > 1 && sc > 0 && pipe_fits(h, nmax, false);
+  bool forced = false;
+  for (const char* e : {"GPE_TILE_X", "GPE_SEG_X", "GPE_SEG_YZ", "GPE_KEEP", "GPE_PIPE", "GPE_FUSE_XY"})
+    forced = forced || std::getenv(e);
+  if (h->dim == 3 && h->geom == 0 && !forced) choose_shapes_3d(h);
 }
 
 }  // namespace

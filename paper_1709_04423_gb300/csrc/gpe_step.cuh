@@ -394,6 +394,9 @@ inline bool strang_close_fused(const gp_handle* h, bool imag) {
 //  * FP32 y/z, fewer than 64 tiles of 32-point segments (lines over 258 points):
 //    512^2 imaginary 11.7 -> 5.2; 257 x 201 (16-point ones) would lose, 4.2 -> 5.4,
 //    to the staging through shared memory;
+//  * double-float 3d, lines over 130 points, in segments of 8 instead of 16 or 32:
+//    160 x 144 x 150 imaginary 122 / 58 / 67 -> 89 / 47 / 57, real 186 / 85 / 82 ->
+//    125 / 71 / 68 (its long dependent chains want more threads per line);
 //  * double-float x, fewer than 64 tiles: 257 x 201 37.8 -> 29.9; y would lose,
 //    19.0 -> 20.5.
 // The plan picks the segments' length on 2d grids in imaginary time and on axial
@@ -408,13 +411,15 @@ FlexPlan flex_sweep(const gp_handle* h, bool imag, int d, int seg) {
   if (seg > 0) {
     if (d == 0 ? h->pipe_x || h->tma_x : h->pipe_c || h->tma_c) return FlexPlan();
     if (d < 2 && xy_fused(h)) return FlexPlan();
-    if (d > 0 || h->tile_x) {
+    if (d == 0 && !h->tile_x) seg = tile_seg(n - 2);
+    if (is_df<T>::value && h->dim == 3 && seg >= 16) {
+      seg = 8;  // (more, shorter segments: see above)
+    } else if (d > 0 || h->tile_x) {
       const long tiles = (nlines + 31) / 32;
       if (tiles >= (std::is_same<T, double>::value ? 96 : 64)) return FlexPlan();
       if (d > 0 && std::is_same<T, float>::value && seg < 32) return FlexPlan();
     }
     if (h->dim == 2 && (imag || h->geom == 2)) seg = 0;
-    else if (d == 0 && !h->tile_x) seg = tile_seg(n - 2);
   } else if (!imag) {
     seg = tile_seg(n - 2);  // (0 for the lines over 514 points)
   }
