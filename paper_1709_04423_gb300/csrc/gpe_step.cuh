@@ -242,6 +242,7 @@ unsigned launch_tc(gp_handle* h, const Sweep2Args<float>& a, cudaStream_t s, boo
   T.limit_ns = h->tma_limit_ns;
   T.expect_extra = h->tma_expect_extra;
   T.err = h->dev_err;
+  T.last_first = g.axis == 1;
   T.depth = 0;  // (x sweep only)
   int per_sm = 0, sms = 0, dev = 0;
   cudaGetDevice(&dev);
@@ -299,6 +300,7 @@ unsigned launch_tx(gp_handle* h, Sweep2Args<float> a, int mode, cudaStream_t s, 
   T.limit_ns = h->tma_limit_ns;
   T.expect_extra = h->tma_expect_extra;
   T.err = h->dev_err;
+  T.last_first = false;
   T.depth = std::max(1, h->even_depth[mode][si]);
   int per_sm = 0, sms = 0, dev = 0;
   cudaGetDevice(&dev);

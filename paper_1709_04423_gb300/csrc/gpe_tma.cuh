@@ -132,6 +132,7 @@ struct TmaTiles {
   unsigned long long limit_ns;  // bound of every mbarrier wait
   int expect_extra;  // bytes added to every expected transaction count (0; a test sets it to make a wait run out)
   int* err;          // device error flag (GPE_TMA_ERR_*), 0 = fine
+  bool last_first;   // y sweep: tiles in descending order, see tmacol_kernel
   int depth;         // x sweep: segments whose carries reach a segment (the others' tables are below 2^-48)
 };
 
@@ -365,6 +366,11 @@ __device__ __forceinline__ void tma_producer(const TmaTiles& T, unsigned full0, 
 // consumer warps (warp = segment) and one producer warp; dynamic shared
 // memory: the coefficients (3n + 512 complex), then, from the next 1024-byte
 // boundary, kTmaStages tiles of 32 n complex values.
+// The x sweep before a y sweep goes through the xy planes in ascending order and
+// leaves the last of them in L2; the y sweep starts with those (last_first), so
+// that they are read, and overwritten before they are written back, from there:
+// 256^3 (134 MB in a 129 MB L2) 148.8 -> 141.9 us per step in real time, 154.1 ->
+// 145.1 in imaginary time; 56 MB states are all hits either way.
 template <bool IMAG, bool LAST, int SEG, bool CLOSE>
 __global__ void __launch_bounds__(544, 1) tmacol_kernel(const __grid_constant__ CUtensorMap tm, Sweep2Args<float> A,
                                                         TmaTiles T) {
@@ -383,6 +389,7 @@ __global__ void __launch_bounds__(544, 1) tmacol_kernel(const __grid_constant__ 
   float2* tiles = reinterpret_cast<float2*>(tma_smem_raw + (tiles0 - base));
   const bool yaxis = G.axis == 1;
   auto coords = [&](int t, int& c0, int& c1, int& c2) {
+    if (T.last_first) t = T.ntiles - 1 - t;
     const int ix = t % T.nxt, oc = t / T.nxt;
     c0 = ix * 32;
     c1 = yaxis ? 0 : oc;
