@@ -94,29 +94,29 @@ __device__ __forceinline__ df64 line_rsqrt(df64 s) {
 }
 
 // The pending factor 1/sqrt(wscale * total) from the warps' norm sums in
-// shared memory, by every warp for itself: FP64 sums for an FP64 state,
-// double-float ones (48 bits, on the FP32 pipes: a warp's FP64 chain would
-// take longer than the rest of the step) for the others.
+// shared memory, by every warp for itself.  The sums are added in the state
+// precision (as a block's are in the other kernels), the factor is formed in
+// FP64 for an FP64 state and in double-float for the others (48 bits, on the
+// FP32 pipes: a warp's FP64 chain would take longer than the rest of the step).
 template <typename T>
-__device__ __forceinline__ T line_factor(const T* nrm, int nparts, double wscale) {
-  using R = typename std::conditional<std::is_same<T, double>::value, double, df64>::type;
+using line_scale_t = typename std::conditional<std::is_same<T, double>::value, double, df64>::type;
+
+template <typename T>
+__device__ __forceinline__ T line_factor(const T* nrm, int nparts, line_scale_t<T> ws) {
   const int lane = threadIdx.x & 31;
-  R s = R(0);
-  for (int i = lane; i < nparts; i += 32) {
-    if constexpr (std::is_same<T, float>::value) s = s + df64(nrm[i], 0.f);
-    else s = s + nrm[i];
-  }
+  T s = T(0);
+  for (int i = lane; i < nparts; i += 32) s = s + nrm[i];
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1)
     if (o < nparts) s = s + shfl_xor_t(s, o);
   // (with fewer parts than lanes only the low lanes hold sums)
   if constexpr (std::is_same<T, double>::value) {
-    return line_rsqrt(__shfl_sync(0xffffffffu, s, 0) * wscale);
+    return line_rsqrt(__shfl_sync(0xffffffffu, s, 0) * ws);
+  } else if constexpr (std::is_same<T, float>::value) {
+    return line_rsqrt(dfl::df_mulf(ws, __shfl_sync(0xffffffffu, s, 0))).hi;
   } else {
     const df64 t = df64(__shfl_sync(0xffffffffu, s.hi, 0), __shfl_sync(0xffffffffu, s.lo, 0));
-    const df64 f = line_rsqrt(t * df64(wscale));
-    if constexpr (std::is_same<T, float>::value) return f.hi;
-    else return f;
+    return line_rsqrt(t * ws);
   }
 }
 
@@ -243,11 +243,12 @@ __global__ void __launch_bounds__(kLineMaxThreads) line_steps_kernel(const __gri
     if (threadIdx.x == 0) s_z[W] = zero;  // in this block's copy: nothing comes after the last warp
   }
 
+  const line_scale_t<T> ws(A.parts_wscale);
   T nval = T(0);
   for (long t = 0; t < P.nsteps; ++t) {
     // ---- the pending renormalisation and N
     if (IMAG && t > 0) {
-      const T scl = line_factor<T>(s_nrm, W, A.parts_wscale);
+      const T scl = line_factor<T>(s_nrm, W, ws);
 #pragma unroll
       for (int j = 0; j < S; ++j) {
         p[j].x = p[j].x * scl;
@@ -391,7 +392,7 @@ __global__ void __launch_bounds__(kLineMaxThreads) line_steps_kernel(const __gri
     }
   }
   if (IMAG) {
-    const T scl = line_factor<T>(s_nrm, W, A.parts_wscale);
+    const T scl = line_factor<T>(s_nrm, W, ws);
 #pragma unroll
     for (int j = 0; j < S; ++j) {
       p[j].x = p[j].x * scl;
