@@ -474,7 +474,14 @@ bool enqueue_sweep(gp_handle* h, bool imag, NormSlots ns, int d, const void* src
     }
     bool done = false;
     if (flex.threads > 0) {
-      run_flex<T>(a, flex, imag, write, fuse_close, var, h->work, h->pdl_now);
+      // Programmatic launches place a sweep's first blocks wherever the previous
+      // one leaves room, so that some SMs take two of its one and a half blocks per
+      // SM more than others: with the heavy blocks of long lines and of
+      // double-float that costs more than the launch it hides (1000 x 1000 FP32
+      // imaginary 40.4 us per step with, 30.7 without; 400 x 300 double-float real
+      // 66.6 and 58.0; but 128 x 128 FP32 8.6 and 10.1).
+      const bool pdl = h->pdl_now && !is_df<T>::value && axis_len(h, d) <= 514;
+      run_flex<T>(a, flex, imag, write, fuse_close, var, h->work, pdl);
       count_launch();
       blocks = flex.blocks;
       if (write && blocks > kFoldParts) {
