@@ -374,7 +374,7 @@ int gp_observables_noalloc(int dim, const int n[3], const double dx[3], const do
  * y/z input segment is kept in registers or streamed and read again, and
  * whether the x and y/z sweeps run as persistent double-buffered kernels
  * (possible where two 32-line tiles fit in shared memory); shape 0 means the
- * thread-per-line kernels used for lines longer than 514 points.  Defaults are set by
+ * general kernels used for lines longer than 514 points.  Defaults are set by
  * gp_init.  gp_autotune times every valid shape of the x sweep and of the y/z
  * sweeps on this handle's grid (2 warm-up + nsteps timed steps each, imaginary
  * time if imag != 0; 1 <= nsteps <= 256), keeps the fastest, restores the

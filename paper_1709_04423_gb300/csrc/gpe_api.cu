@@ -372,7 +372,8 @@ int env_int(const char* name, int dflt) {
 // most 16 segments: seg = smallest of 4, 8, 16, 32 with ceil((n-2)/seg) <= 16.
 // x lines in 2d/3d: the shared-memory tile kernel with the same rule; the 1d
 // line: one warp per line with 32 * seg_x >= n - 2.  Lines longer than 514
-// points use the thread-per-line kernel (shape 0).  GPE_SEG_X, GPE_SEG_YZ and
+// points have no such shape (0): they take tiles of few lines (gpe_flex.cuh), 1d
+// runs gpe_line.cuh, and only lines too long for those the thread-per-line kernel.  GPE_SEG_X, GPE_SEG_YZ and
 // GPE_TILE_X override the defaults (used by the autotuner and the shape tests).
 // two shared-memory stages of a 32-line tile plus the coefficient tables
 // (200 KB of dynamic shared memory leaves room for the kernel's static carry

@@ -113,12 +113,12 @@ struct gp_handle {
   // coefficients, forward right-hand-side factors and stencil factors
   // (vab, vbf, vh of Sweep2Args; 3 n[0] complex values)
   void* cvar[gpe::NUM_MODES] = {nullptr};
-  // legacy thread-per-line factors (m_k, c'_k) per (imag, axis), used when a
+  // thread-per-line factors (m_k, c'_k) per (imag, axis), used when a
   // line is too long for the segmented kernels
   void* cm[2][3] = {{nullptr}};
   void* ccp[2][3] = {{nullptr}};
-  // kernel shapes: segment length per x / y,z lines (0 = thread-per-line
-  // kernel) and whether the x lines are staged through a shared-memory tile
+  // kernel shapes: segment length per x / y,z lines (0 = more than
+  // 514 points: gpe_flex.cuh, else the thread-per-line kernel) and whether the x lines are staged through a shared-memory tile
   int seg_x = 0, seg_c = 0;
   bool tile_x = false;
   int keep_c = 1;  // y/z sweeps keep their input segment in registers (when short enough)

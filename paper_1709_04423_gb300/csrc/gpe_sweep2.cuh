@@ -41,7 +41,9 @@
 //    coalesced accesses and transposed into shared memory (pitch 33), the
 //    sub-step N and the pending renormalisation are applied on the way in
 //    (FIRST), the segments are solved as above, and the tile is written back.
-//  * x line in 1d: one warp per line, lane = segment, carries by shuffles.
+//  * x line in 1d, one sweep at a time: one warp per line, lane = segment, carries
+//    by shuffles (whole runs: gpe_line.cuh).
+// Grids of few lines and lines of more than 514 points: gpe_flex.cuh.
 // LAST (imaginary time) accumulates the Simpson-weighted norm of the output:
 // each thread and then each block sums in the state precision, the per-block
 // totals are summed over the grid in FP64 in a fixed order, and the last block
@@ -212,7 +214,7 @@ __device__ __forceinline__ c2_t<T> phase_N(c2_t<T> p, c2_t<T> F, T dtg) {
 // (exp(-th) - 1) p.  The coefficients are Taylor series -- for |th| < 1/32 sin to
 // th^7, cos - 1 to th^8, exp - 1 to th^8, for |th| < 1/4 to th^11, th^12, th^12
 // (first omitted terms below 1e-17 of the coefficient) -- else the library
-// functions.  A rounded factor next to 1 (F above) repeats its own rounding at a
+// functions.  A rounded factor next to 1 (phase_N's F) repeats its own rounding at a
 // point step after step; here only the small coefficient is rounded, and the
 // sum's rounding is unbiased.  19 FP64 operations per point against 24 in real
 // time, 13 against 15 in imaginary time.
