@@ -309,7 +309,11 @@ __device__ __forceinline__ void flex_body(const Sweep2Args<T>& A, const FlexTile
     if (s < F.nseg) cbv[slot(s)] = z[0];
   }
   __syncthreads();
+  // FP32 states on grids with lines over 514 points (A.norm64): a thread's squares
+  // as SquareSum does, FP64 from there on
+  constexpr bool kNorm64 = LAST && !CLOSE && std::is_same<T, float>::value;
   T nval = T(0);
+  [[maybe_unused]] double nval64 = 0.0;
   if (solving) {
     V Zin = vzero;
     if (small) {
@@ -359,7 +363,23 @@ __device__ __forceinline__ void flex_body(const Sweep2Args<T>& A, const FlexTile
         }
         if (j < jm && solver) {
           if (GPE_CHECK(base + (long)k * st < lim, 303)) X::set(line[(long)k * st], comp, u);
-          if (LAST) tacc += A.w_axis[k] * X::sq(u);
+          if (LAST && !(kNorm64 && A.norm64)) tacc += A.w_axis[k] * X::sq(u);
+        }
+        if constexpr (kNorm64) z[j] = u;
+      }
+      if constexpr (kNorm64) {
+        if (A.norm64 && solver) {
+          SquareSum sum;
+#pragma unroll
+          for (int j = 0; j < SEG; ++j) sum.peak(z[j].x, z[j].y);  // (zeros past the line's end)
+          sum.scale();
+#pragma unroll
+          for (int j = 0; j < SEG; ++j) {
+            const float w = j < jm ? A.w_axis[k0 + j] : 0.f;
+            sum.add(w, z[j].x);
+            sum.add(w, z[j].y);
+          }
+          nval64 = sum.total() * ((double)A.w_a[ci] * A.w_b[cf2]);
         }
       }
       if (s == 0 && solver && GPE_CHECK(base + (long)(n - 1) * st < lim, 304)) {
@@ -376,6 +396,14 @@ __device__ __forceinline__ void flex_body(const Sweep2Args<T>& A, const FlexTile
       const int cc = i / per_line, k = (i - cc * per_line) * 32 + lane;
       if (k < n && GPE_CHECK((long)(L0 + cc) * G.nx + k < lim, 305))
         A.psi[(long)(L0 + cc) * G.nx + k] = (k >= 1 && k <= M) ? at(cc, k) : zero;
+    }
+  }
+  if constexpr (kNorm64) {
+    if (A.norm64) {
+      double v[1] = {nval64};
+      block_sum<1>(v, red_smem);
+      if (tid == 0) A.parts_out[blockIdx.x] = v[0];
+      return;
     }
   }
   finish_norm<T, LAST>(nval, A.parts_out);

@@ -93,11 +93,17 @@ __device__ __forceinline__ df64 line_rsqrt(df64 s) {
   return df64(y0, 0.f) + dfl::df_mulf(dfl::df_scale(r, 0.5f) + df64(0.375f * r.hi * r.hi, 0.f), y0);
 }
 
+// The type a line's norm is summed in: the state precision (as a block's sums
+// are in the other kernels), and FP64 from each thread's SquareSum on for FP32
+// lines of more than 514 points, the ones with several points per thread (as on
+// the long lines of 2d and 3d grids; see flex_body).
+template <typename T, int S>
+using line_norm_t = typename std::conditional<std::is_same<T, float>::value && (S > 1), double, T>::type;
+
 // The pending factor 1/sqrt(wscale * total) from the warps' norm sums in
-// shared memory, by every warp for itself.  The sums are added in the state
-// precision (as a block's are in the other kernels), the factor is formed in
-// FP64 for an FP64 state and in double-float for the others (48 bits, on the
-// FP32 pipes: a warp's FP64 chain would take longer than the rest of the step).
+// shared memory, by every warp for itself: in FP64 from FP64 sums, in
+// double-float from the others (48 bits, on the FP32 pipes: a warp's FP64 chain
+// would take longer than the rest of the step).
 template <typename T>
 using line_scale_t = typename std::conditional<std::is_same<T, double>::value, double, df64>::type;
 
@@ -125,7 +131,8 @@ __global__ void __launch_bounds__(kLineMaxThreads) line_steps_kernel(const __gri
   using c2 = c2_t<T>;
   __shared__ c2 s_first[kLineMaxWarps], s_last[kLineMaxWarps], s_end[kLineMaxWarps], s_z[kLineMaxWarps + 1];
   __shared__ c2 s_A[kLineMaxWarps], s_B[kLineMaxWarps], s_cr[kLineMaxWarps];
-  __shared__ T s_nrm[kLineMaxWarps];
+  using NT = line_norm_t<T, S>;
+  __shared__ NT s_nrm[kLineMaxWarps];
   const Sweep2Args<T>& A = P.a;
   const int n = A.geom.n, M = n - 2;
   const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
@@ -243,12 +250,11 @@ __global__ void __launch_bounds__(kLineMaxThreads) line_steps_kernel(const __gri
     if (threadIdx.x == 0) s_z[W] = zero;  // in this block's copy: nothing comes after the last warp
   }
 
-  const line_scale_t<T> ws(A.parts_wscale);
-  T nval = T(0);
+  const line_scale_t<NT> ws(A.parts_wscale);
   for (long t = 0; t < P.nsteps; ++t) {
     // ---- the pending renormalisation and N
     if (IMAG && t > 0) {
-      const T scl = line_factor<T>(s_nrm, W, ws);
+      const T scl = (T)line_factor<NT>(s_nrm, W, ws);
 #pragma unroll
       for (int j = 0; j < S; ++j) {
         p[j].x = p[j].x * scl;
@@ -382,9 +388,22 @@ __global__ void __launch_bounds__(kLineMaxThreads) line_steps_kernel(const __gri
 #pragma unroll
         for (int j = 0; j < S; ++j) p[j] = phase(p[j], j);
       }
-      nval = T(0);
+      NT nval = NT(0);
+      if constexpr (std::is_same<NT, T>::value) {
 #pragma unroll
-      for (int j = 0; j < S; ++j) nval = nval + wk[j] * (p[j].x * p[j].x + p[j].y * p[j].y);
+        for (int j = 0; j < S; ++j) nval = nval + wk[j] * (p[j].x * p[j].x + p[j].y * p[j].y);
+      } else {
+        SquareSum sum;
+#pragma unroll
+        for (int j = 0; j < S; ++j) sum.peak(p[j].x, p[j].y);
+        sum.scale();
+#pragma unroll
+        for (int j = 0; j < S; ++j) {
+          sum.add(wk[j], p[j].x);
+          sum.add(wk[j], p[j].y);
+        }
+        nval = sum.total();
+      }
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) nval = nval + shfl_xor_t(nval, o);
       if (C > 1 || lane == 0) publish(s_nrm, w, nval);
@@ -392,7 +411,7 @@ __global__ void __launch_bounds__(kLineMaxThreads) line_steps_kernel(const __gri
     }
   }
   if (IMAG) {
-    const T scl = line_factor<T>(s_nrm, W, ws);
+    const T scl = (T)line_factor<NT>(s_nrm, W, ws);
 #pragma unroll
     for (int j = 0; j < S; ++j) {
       p[j].x = p[j].x * scl;
@@ -418,8 +437,9 @@ __global__ void __launch_bounds__(kLineMaxThreads) line_steps_kernel(const __gri
 // where the measured step times cross (us per step):
 //  * FP32: one block's barriers are cheaper than a cluster's, so a second block
 //    only from 512 threads of 4 points on (513 points, imaginary time: 1.58 with
-//    one block, 2.02 with four; 1000 real: 1.17 against 1.50; 4001 imaginary:
-//    2.58 with four blocks of 256 threads, 3.22 with two of 512);
+//    one block, 2.02 with four; 1000 real: 1.17 against 1.50; 4001 imaginary,
+//    before its norm's FP64 part: 2.58 with four blocks of 256 threads, 3.22 with
+//    two of 512; 4.22 now);
 //  * FP64 is bound by its two FP64 lanes per SM and the latency of its chain,
 //    so about 64 points per block (256 points: 5.63 with one block, 3.92 with
 //    four; 1000: 4.63 with eight, 6.81 with four), and more than one point per

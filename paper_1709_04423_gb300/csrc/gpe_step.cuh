@@ -464,6 +464,7 @@ bool enqueue_sweep(gp_handle* h, bool imag, NormSlots ns, int d, const void* src
     a.w_a = (const T*)(d == 0 ? h->wt[1] : h->wt[0]);
     a.w_b = (const T*)(d == 2 ? h->wt[1] : h->wt[2]);
     a.parts_out = parts_out;
+    a.norm64 = d > 0 && h->seg_c == 0;
     // the rho axis of a circular or axial trap: non-symmetric coefficients
     const bool var = h->geom == 2 && d == 0;
     if (var) {
