@@ -142,7 +142,13 @@ int gp_init_axial(gp_handle** out, int n_rho, int n_z, double drho, double dz, d
 int gp_set_state(gp_handle* h, const void* psi, int on_device);
 
 /* Copies the state out in the handle's precision (GP_DF64: rounded to
- * double).  With on_device == 0 the call synchronises the stream. */
+ * double).  With on_device == 0 the call synchronises the stream and, like
+ * every call that does, returns GP_ERR_TIMEOUT if a bounded device-side wait
+ * of an earlier step gave up (the TMA sweeps, see GP_SHAPE_TMA_YZ; large FP32
+ * grids take them by default).  With on_device != 0 the copy is asynchronous
+ * and cannot report that: the array is then filled with NaN instead (so are
+ * the device outputs of gp_reduced_density and gp_step_series), and the error
+ * stays for the next synchronising call. */
 int gp_get_state(gp_handle* h, void* psi, int on_device);
 
 /* Replaces the harmonic trap by a potential array (double, npoints values);
@@ -394,8 +400,8 @@ int gp_observables_noalloc(int dim, const int n[3], const double dx[3], const do
  * global and shared memory with the TMA unit, three stages deep, and solve
  * them in place with the same per-line arithmetic as the other y/z sweeps.
  * Their waits for a tile give up after a limit (1 s, or GPE_WAIT_LIMIT_MS
- * milliseconds at gp_init); the next synchronising call (gp_observables) then
- * returns GP_ERR_TIMEOUT.
+ * milliseconds at gp_init); the next synchronising call (gp_observables, a
+ * read to the host) then returns GP_ERR_TIMEOUT.
  * GP_SHAPE_TMA_X (GP_F32 complex states of Cartesian 2d/3d grids with nx a
  * multiple of 16 and at most 256, the x tile with seg_x 8 or 16): the x sweep,
  * with the sub-step N and the pending renormalisation, runs the same way, its
@@ -446,7 +452,7 @@ int gp_check_status(int* first_failure);
  * (GP_SHAPE_TMA_X / GP_SHAPE_TMA_YZ) announces extra_bytes more than it
  * moves, so its wait on the tile can never complete: each such sweep gives up
  * after the wait limit (GPE_WAIT_LIMIT_MS at gp_init, default 1000 ms), and
- * the next gp_observables returns GP_ERR_TIMEOUT -- the way the tests check
+ * the next synchronising call returns GP_ERR_TIMEOUT -- the way the tests check
  * that a wait that runs out ends the kernel and leaves the context usable.
  * 0 restores normal operation; the state is not valid after a timeout
  * (set it again).  0 <= extra_bytes <= 1024, else GP_ERR_INVALID. */

@@ -426,14 +426,35 @@ bool tma_x_fits(const gp_handle* h, int seg) {
   return smem + 17 * 1024 <= 227L * 1024;  // + the static carries, edge points and barriers
 }
 
+int fetch_dev_err(gp_handle* h) {
+  if (h->tma_used) GP_CUDA(cudaMemcpyAsync(h->obs_host + 8, h->dev_err, sizeof(int), cudaMemcpyDeviceToHost, h->work));
+  return GP_OK;
+}
+
 int read_dev_err(gp_handle* h, const char* who) {
-  GP_CUDA(cudaMemcpyAsync(h->obs_host + 8, h->dev_err, sizeof(int), cudaMemcpyDeviceToHost, h->work));
+  const int rc = fetch_dev_err(h);
+  if (rc) return rc;
   GP_CUDA(cudaStreamSynchronize(h->work));
   return take_dev_err(h, who);
 }
 
-// The device error flag that a transfer has brought to obs_host[8].
+namespace {
+__global__ void void_on_err_kernel(unsigned* out, long n, const int* err) {
+  if (*err == 0) return;
+  for (long q = (long)blockIdx.x * blockDim.x + threadIdx.x; q < n; q += (long)gridDim.x * blockDim.x) out[q] = ~0u;
+}
+}  // namespace
+
+void void_on_dev_err(gp_handle* h, void* out, size_t bytes) {
+  if (!h->tma_used) return;
+  const long n = (long)(bytes / sizeof(unsigned));
+  const int blocks = (int)std::min<long>((n + 255) / 256, 152);
+  void_on_err_kernel<<<blocks, 256, 0, h->work>>>((unsigned*)out, n, h->dev_err);
+  count_launch();
+}
+
 int take_dev_err(gp_handle* h, const char* who) {
+  if (!h->tma_used) return GP_OK;
   int e = 0;
   std::memcpy(&e, h->obs_host + 8, sizeof(int));
   if (e == 0) return GP_OK;
@@ -912,8 +933,9 @@ int gp_get_state(gp_handle* h, void* psi, int on_device) {
     materialize_complex(h);  // a real state: its complex copy
     GP_CUDA(cudaMemcpyAsync(psi, h->psi, (size_t)h->np * h->esize,
                             on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, h->work));
+    if (on_device) void_on_dev_err(h, psi, (size_t)h->np * h->esize);
   }
-  if (!on_device) GP_CUDA(cudaStreamSynchronize(h->work));
+  if (!on_device && (rc = read_dev_err(h, "gp_get_state"))) return rc;
   return join_out(h);
 }
 
@@ -1045,7 +1067,8 @@ int gp_time_sweeps(gp_handle* h, int imag, long nsteps, double* ms_per_launch) {
   if (!h || !ms_per_launch) return fail(GP_ERR_INVALID, "gp_time_sweeps: NULL argument");
   if (nsteps < 0 || nsteps > 4096) return fail(GP_ERR_INVALID, "gp_time_sweeps: nsteps must be in [0, 4096]");
   if (h->real_mode && !imag) return fail(GP_ERR_STATE, "gp_time_sweeps: a real state takes imaginary-time steps only");
-  return time_steps_any(h, imag != 0, nsteps, ms_per_launch);
+  const int rc = time_steps_any(h, imag != 0, nsteps, ms_per_launch);
+  return rc ? rc : read_dev_err(h, "gp_time_sweeps");
 }
 
 namespace {
@@ -1123,7 +1146,7 @@ int gp_adjoint_backward(gp_handle* h, const void* lambda_T, int lambda_on_device
   if (dJdV && !dJdV_on_device)
     GP_CUDA(cudaMemcpyAsync(dJdV, h->adj_dJdV, (size_t)h->np * sizeof(double), cudaMemcpyDeviceToHost, h->work));
   GP_CUDA(cudaMemcpyAsync(h->obs_host, h->adj_dJdg, sizeof(double), cudaMemcpyDeviceToHost, h->work));
-  GP_CUDA(cudaStreamSynchronize(h->work));
+  if ((rc = read_dev_err(h, "gp_adjoint_backward"))) return rc;
   if ((rc = join_out(h))) return rc;
   if (dJdg) *dJdg = h->obs_host[0];
   if (!std::isfinite(h->obs_host[0])) return fail(GP_ERR_NONFINITE, "gp_adjoint_backward: non-finite gradient");
@@ -1423,10 +1446,11 @@ int gp_step_series(gp_handle* h, int imag, long nsteps, int every, double* out, 
     const int blocks = (int)std::min<long>((nrec + 127) / 128, 152L * 4);
     series_finish_kernel<<<blocks, 128, 0, h->work>>>(h->series_buf, nrec, h->g, dst);
     count_launch();
+    if (out_on_device) void_on_dev_err(h, out, 7 * (size_t)nrec * sizeof(double));
     GP_CUDA(cudaGetLastError());
     if (!out_on_device) {
       GP_CUDA(cudaMemcpyAsync(out, dst, 7 * (size_t)nrec * sizeof(double), cudaMemcpyDeviceToHost, h->work));
-      GP_CUDA(cudaStreamSynchronize(h->work));
+      if ((rc = read_dev_err(h, "gp_step_series"))) return rc;
     }
   }
   return join_out(h);

@@ -129,6 +129,7 @@ struct gp_handle {
   // (gpe_tma.cuh); their mbarrier waits give up after tma_limit_ns and then
   // set *dev_err, which the next synchronising call turns into GP_ERR_TIMEOUT
   bool tma_c = false;
+  bool tma_used = false;  // a sweep with such waits has been launched
   bool tma_x = false;  // the x sweep too (FP32, nx a multiple of 16, at most 256)
   int* dev_err = nullptr;
   unsigned long long tma_limit_ns = 1000000000ull;
@@ -218,8 +219,16 @@ int tile_seg(int M);
 bool plane_fits(const gp_handle* h, int seg);  // the fused x + y sweep kernel takes this grid and segment length
 bool tma_fits(const gp_handle* h, int seg);    // the TMA y/z sweeps take this grid and segment length
 bool tma_x_fits(const gp_handle* h, int seg);  // the TMA x sweep takes this grid and segment length
+// Whether a device wait of this handle's sweeps gave up: fetch_dev_err enqueues the
+// flag's copy to the host, take_dev_err reads it once the stream has been
+// waited for (GP_ERR_TIMEOUT, and clears it), read_dev_err does both.  A result
+// that stays on the device cannot be reported so: void_on_dev_err enqueues a
+// kernel that fills it with NaN (all bits set) if the flag is set.  Only
+// handles that have launched a sweep with such waits (tma_used) need either.
+int fetch_dev_err(gp_handle* h);
 int take_dev_err(gp_handle* h, const char* who);
-int read_dev_err(gp_handle* h, const char* who);  // GP_ERR_TIMEOUT (and clears it) if a device wait gave up
+int read_dev_err(gp_handle* h, const char* who);
+void void_on_dev_err(gp_handle* h, void* out, size_t bytes);
 
 int dev_alloc(gp_handle* h, void** p, size_t bytes);
 // Device buffers of handles and batches: cudaMalloc / cudaFree, and in the

@@ -150,10 +150,11 @@ extern "C" int gp_reduced_density(gp_handle* h, int keep_mask, double* out, int 
   else
     reduce_stage2<<<(unsigned)((G.nout + 255) / 256), 256, 0, h->work>>>(h->red_parts, G, dout);
   count_launch();
+  if (out_on_device) void_on_dev_err(h, out, (size_t)G.nout * sizeof(double));
   GP_CUDA(cudaGetLastError());
   if (!out_on_device) {
     GP_CUDA(cudaMemcpyAsync(out, dout, (size_t)G.nout * sizeof(double), cudaMemcpyDeviceToHost, h->work));
-    GP_CUDA(cudaStreamSynchronize(h->work));
+    if ((rc = read_dev_err(h, "gp_reduced_density"))) return rc;
   }
   return join_out(h);
 }

@@ -239,6 +239,7 @@ unsigned launch_tc(gp_handle* h, const Sweep2Args<float>& a, cudaStream_t s, boo
   TmaTiles T;
   T.nxt = (g.nx + 31) / 32;
   T.ntiles = T.nxt * (g.axis == 1 ? g.nz : g.ny);
+  h->tma_used = true;
   T.limit_ns = h->tma_limit_ns;
   T.expect_extra = h->tma_expect_extra;
   T.err = h->dev_err;
@@ -297,6 +298,7 @@ unsigned launch_tx(gp_handle* h, Sweep2Args<float> a, int mode, cudaStream_t s, 
   TmaTiles T;
   T.nxt = 1;
   T.ntiles = (int)((g.nlines + 31) / 32);
+  h->tma_used = true;
   T.limit_ns = h->tma_limit_ns;
   T.expect_extra = h->tma_expect_extra;
   T.err = h->dev_err;
