@@ -458,6 +458,12 @@ int gp_check_status(int* first_failure);
  * (set it again).  0 <= extra_bytes <= 1024, else GP_ERR_INVALID. */
 int gp_test_stall_transfers(gp_handle* h, int extra_bytes);
 
+/* Test hook of the TMA sweeps' tensor maps.  With refuse = 1 this handle's maps
+ * count as refused by the driver: the step, timing or adjoint call that needs
+ * one returns GP_ERR_CUDA, and the state is not valid (set it again).  0
+ * restores normal operation.  Any other value: GP_ERR_INVALID. */
+int gp_test_refuse_maps(gp_handle* h, int refuse);
+
 /* Test hook of the one-launch batch form's bounded step waits (the paper has
  * no counterpart).  With extra > 0 every wait of mode 1 asks for extra more
  * finished items than the launch will ever count, so the first y sweep's

@@ -431,6 +431,13 @@ int fetch_dev_err(gp_handle* h) {
   return GP_OK;
 }
 
+int take_launch_err(gp_handle* h) {
+  if (h->launch_err.empty()) return GP_OK;
+  const std::string msg = h->launch_err + "; the state is not valid";
+  h->launch_err.clear();
+  return fail(GP_ERR_CUDA, msg);
+}
+
 int read_dev_err(gp_handle* h, const char* who) {
   const int rc = fetch_dev_err(h);
   if (rc) return rc;
@@ -1232,6 +1239,14 @@ int gp_test_stall_transfers(gp_handle* h, int extra_bytes) {
     return fail(GP_ERR_INVALID, "gp_test_stall_transfers: extra_bytes must be in [0, 1024]");
   drop_graphs(h);  // captured launches carry the old value
   h->tma_expect_extra = extra_bytes;
+  return GP_OK;
+}
+
+int gp_test_refuse_maps(gp_handle* h, int refuse) {
+  if (!h) return fail(GP_ERR_INVALID, "gp_test_refuse_maps: NULL handle");
+  if (refuse != 0 && refuse != 1) return fail(GP_ERR_INVALID, "gp_test_refuse_maps: refuse must be 0 or 1");
+  drop_graphs(h);  // captured launches carry their maps
+  h->tma_refuse = refuse != 0;
   return GP_OK;
 }
 

@@ -130,6 +130,8 @@ struct gp_handle {
   // set *dev_err, which the next synchronising call turns into GP_ERR_TIMEOUT
   bool tma_c = false;
   bool tma_used = false;  // a sweep with such waits has been launched
+  bool tma_refuse = false;  // a test's way to have the tensor maps refused
+  std::string launch_err;   // a sweep that could not be launched (take_launch_err)
   bool tma_x = false;  // the x sweep too (FP32, nx a multiple of 16, at most 256)
   int* dev_err = nullptr;
   unsigned long long tma_limit_ns = 1000000000ull;
@@ -227,6 +229,9 @@ bool tma_x_fits(const gp_handle* h, int seg);  // the TMA x sweep takes this gri
 // handles that have launched a sweep with such waits (tma_used) need either.
 int fetch_dev_err(gp_handle* h);
 int take_dev_err(gp_handle* h, const char* who);
+// GP_ERR_CUDA (and clears it) if a sweep enqueued since the last call could not
+// be launched; the state is then not valid
+int take_launch_err(gp_handle* h);
 int read_dev_err(gp_handle* h, const char* who);
 void void_on_dev_err(gp_handle* h, void* out, size_t bytes);
 

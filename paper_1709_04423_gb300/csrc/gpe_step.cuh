@@ -232,8 +232,8 @@ unsigned launch_tc(gp_handle* h, const Sweep2Args<float>& a, cudaStream_t s, boo
   auto kern = tmacol_kernel<IMAG, LAST, SEG, CLOSE>;
   opt_in_smem((const void*)kern, smem);
   CUtensorMap map;
-  if (!encode_line_map(&map, a.psi, g)) {
-    g_err = "cuTensorMapEncodeTiled refused the state's tensor map";
+  if (h->tma_refuse || !encode_line_map(&map, a.psi, g)) {
+    h->launch_err = "cuTensorMapEncodeTiled refused the state's tensor map";
     return 0;
   }
   TmaTiles T;
@@ -291,8 +291,8 @@ unsigned launch_tx(gp_handle* h, Sweep2Args<float> a, int mode, cudaStream_t s, 
   a.gb = ev + (size_t)(2 * si + 1) * g.n;
   a.ptab = ev + (size_t)4 * g.n + 512 * si;
   CUtensorMap map;
-  if (!encode_row_map(&map, a.psi, g)) {
-    g_err = "cuTensorMapEncodeTiled refused the state's tensor map";
+  if (h->tma_refuse || !encode_row_map(&map, a.psi, g)) {
+    h->launch_err = "cuTensorMapEncodeTiled refused the state's tensor map";
     return 0;
   }
   TmaTiles T;
@@ -772,6 +772,10 @@ int run_steps_t(gp_handle* h, bool imag, long nsteps) {
         enqueue_step<T>(h, imag, slots_of_step(imag, t + s), nullptr, nullptr, next_f);
       g_launches.store(before);  // capturing launches nothing
       GP_CUDA(cudaStreamEndCapture(h->work, &graph));
+      if ((rc = take_launch_err(h))) {
+        cudaGraphDestroy(graph);
+        return rc;
+      }
       cudaError_t e = cudaGraphInstantiate(&ge, graph, 0);
       cudaGraphDestroy(graph);
       if (e != cudaSuccess) {
@@ -788,6 +792,7 @@ int run_steps_t(gp_handle* h, bool imag, long nsteps) {
   for (; t < nsteps; ++t) enqueue_step<T>(h, imag, slots_of_step(imag, t), nullptr, nullptr, next_f);
   if (merged) enqueue_strang_close<T>(h, false, NormSlots{});
   if (imag) enqueue_finish_imag<T>(h, nsteps);
+  if ((rc = take_launch_err(h))) return rc;
   GP_CUDA(cudaGetLastError());
   return join_out(h);
 }
@@ -803,6 +808,7 @@ int time_steps_t(gp_handle* h, bool imag, long nsteps, double* ms_out) {
   for (long t = 0; t < nsteps && !rc; ++t)
     enqueue_step<T>(h, imag, slots_of_step(imag, t), ev.data() + (size_t)t * 2 * h->dim);
   if (imag && !rc && nsteps > 0) enqueue_finish_imag<T>(h, nsteps);
+  if (!rc) rc = take_launch_err(h);
   cudaError_t e = cudaStreamSynchronize(h->work);
   if (!rc && e != cudaSuccess) rc = fail(GP_ERR_CUDA, std::string("gp_time_sweeps: ") + cudaGetErrorString(e));
   double acc[3] = {0, 0, 0};
@@ -833,6 +839,7 @@ int time_sweeps_graph_t(gp_handle* h, bool imag, int reps, double* ms_out) {
   for (int d = 0; d < 3; ++d) ms_out[d] = 0.0;
   PdlScope pdl_scope(h);
   for (long t = 0; t < 2; ++t) enqueue_step<T>(h, imag, slots_of_step(imag, t));
+  if ((rc = take_launch_err(h))) return rc;
   NormSlots ns;
   if (imag) {
     ns.rd = 1;  // written by step 1 above
@@ -1016,6 +1023,7 @@ int adjoint_forward_t(gp_handle* h, long nsteps, int K) {
       PdlScope pdl(h);
       GP_CUDA(cudaMemcpyAsync(h->adj_traj, h->psi, sbytes, cudaMemcpyDeviceToDevice, h->work));
       enqueue_recorded<T>(h, (int)(nsteps - c * K), true);
+      if ((rc = take_launch_err(h))) return rc;
       GP_CUDA(cudaGetLastError());
       h->adj_traj_seg = c;
     }
@@ -1064,6 +1072,10 @@ int adjoint_backward_t(gp_handle* h, double* dJdV_dev, void* lam0_dev) {
   h->g = g_now;
   h->dt = dt_now;
   h->adj_dJdV = dJdV_keep;
+  if ((rc = take_launch_err(h))) {
+    h->adj_traj_seg = -1;  // (a recomputed segment is not what the buffer should hold)
+    return rc;
+  }
   if (lam0_dev) cudaMemcpyAsync(lam0_dev, h->adj_lam, sbytes, cudaMemcpyDeviceToDevice, h->work);
   GP_CUDA(cudaGetLastError());
   return join_out(h);

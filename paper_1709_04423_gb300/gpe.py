@@ -45,7 +45,7 @@ ABI_SYMBOLS = (
     "gp_autotune", "gp_set_shapes", "gp_get_shapes", "gp_reduced_density", "gp_step_series",
     "gp_init_spherical", "gp_set_splitting", "gp_set_real_state", "gp_init_circular", "gp_init_axial",
     "gp_test_stall_transfers", "gp_time_sweeps_graph", "gp_fp_fma_rates", "gp_check_status",
-    "gp_batch_set_mode", "gp_batch_get_mode", "gp_batch_autotune", "gp_test_batch_stall",
+    "gp_batch_set_mode", "gp_batch_get_mode", "gp_batch_autotune", "gp_test_batch_stall", "gp_test_refuse_maps",
 )
 
 
@@ -105,6 +105,7 @@ def _open(path):
     lib.gp_time_sweeps_graph.argtypes = [_vp, I, I, ctypes.POINTER(D)]
     lib.gp_fp_fma_rates.argtypes = [ctypes.POINTER(D), ctypes.POINTER(D)]
     lib.gp_test_stall_transfers.argtypes = [_vp, I]
+    lib.gp_test_refuse_maps.argtypes = [_vp, I]
     lib.gp_check_status.argtypes = [ctypes.POINTER(I)]
     lib.gp_observables_noalloc.argtypes = [I, ctypes.POINTER(I), ctypes.POINTER(D), ctypes.POINTER(D), D, I,
                                            _vp, _vp, _vp, _vp]
@@ -384,6 +385,11 @@ def gp_test_stall_transfers(h, extra_bytes):
     """Test hook: TMA tile loads announce extra bytes, so their bounded waits
     run out (see include/gpe.h)."""
     return _check(load().gp_test_stall_transfers(h, int(extra_bytes)))
+
+
+def gp_test_refuse_maps(h, refuse):
+    """Test hook: the handle's tensor maps count as refused (see include/gpe.h)."""
+    return _check(load().gp_test_refuse_maps(h, int(refuse)))
 
 
 # ----------------------------------------------------------------- wrapper

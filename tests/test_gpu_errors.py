@@ -81,3 +81,25 @@ def test_a_wait_that_ran_out_leaves_no_results_on_the_device(G, phi0, monkeypatc
     recovers(G, p, phi0)
     assert bool(torch.isfinite(torch.view_as_real(p.get_state(device=True))).all())
     p.close()
+
+
+CALLS = {
+    "step_imag": lambda G, p: p.step_imag(2),
+    "step_real": lambda G, p: p.step_real(40),      # (a captured block of steps among them)
+    "time_sweeps": lambda G, p: p.time_sweeps(True, 1),
+    "time_sweeps_graph": lambda G, p: p.time_sweeps_graph(False, 2),
+    "adjoint": lambda G, p: G.gp_adjoint_forward(p.h, 3, 2),
+    "series": lambda G, p: p.step_series(True, 2, 1),
+}
+
+
+@pytest.mark.parametrize("call", CALLS)
+def test_a_refused_tensor_map_is_an_error(G, phi0, monkeypatch, call):
+    p = default_handle(G, phi0, monkeypatch)
+    G.gp_test_refuse_maps(p.h, 1)
+    with pytest.raises(G.GPError) as e:
+        CALLS[call](G, p)
+    assert e.value.code == G.GP_ERR_CUDA and "tensor map" in str(e.value)
+    G.gp_test_refuse_maps(p.h, 0)
+    recovers(G, p, phi0)
+    p.close()
