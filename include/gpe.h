@@ -419,6 +419,15 @@ int gp_autotune(gp_handle* h, int imag, int nsteps, double* best_ms);
 int gp_set_shapes(gp_handle* h, int tile_x, int seg_x, int seg_c, int flags);
 int gp_get_shapes(const gp_handle* h, int* tile_x, int* seg_x, int* seg_c, int* flags);
 
+/* The kernel that gp_step_imag (imag != 0) or gp_step_real takes for the sweep
+ * along an axis of this handle, a static string: "line" (1d: every step of a
+ * run in one launch), "narrow" (tiles of 1 to 16 lines), "tile" (x: 32-line
+ * tiles), "warp" (x: a warp per line), "column" (y/z: 32 lines per block),
+ * "plane" (x and y fused), "pipelined", "tma", or "thread" (a thread per line).
+ * NULL for a NULL handle, an axis the grid does not have, or real time with a
+ * real state. */
+const char* gp_sweep_kernel(const gp_handle* h, int imag, int axis);
+
 /* Grid queries. */
 long gp_npoints(const gp_handle* h);
 int gp_precision_of(const gp_handle* h);

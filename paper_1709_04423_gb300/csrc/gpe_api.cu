@@ -1305,6 +1305,28 @@ int gp_get_shapes(const gp_handle* h, int* tile_x, int* seg_x, int* seg_c, int* 
   return GP_OK;
 }
 
+const char* gp_sweep_kernel(const gp_handle* h, int imag, int axis) {
+  if (!h || axis < 0 || axis >= h->dim || (h->real_mode && !imag)) return nullptr;
+  SweepKind k;
+  if (h->dim == 1 && (h->prec == GP_DF64 ? takes_line_df(h) : h->prec == GP_F64 ? takes_line_f64(h) : takes_line_f32(h)))
+    k = SWEEP_LINE;
+  else
+    k = h->prec == GP_DF64  ? sweep_kind_df(h, imag != 0, axis)
+        : h->prec == GP_F64 ? sweep_kind_f64(h, imag != 0, axis)
+                            : sweep_kind_f32(h, imag != 0, axis);
+  switch (k) {
+    case SWEEP_LINE: return "line";
+    case SWEEP_NARROW: return "narrow";
+    case SWEEP_PLANE: return "plane";
+    case SWEEP_TMA: return "tma";
+    case SWEEP_PIPE: return "pipelined";
+    case SWEEP_TILE: return "tile";
+    case SWEEP_WARP: return "warp";
+    case SWEEP_COLUMN: return "column";
+    default: return "thread";
+  }
+}
+
 int gp_autotune(gp_handle* h, int imag, int nsteps, double* best_ms) {
   if (!h) return fail(GP_ERR_INVALID, "gp_autotune: NULL handle");
   if (nsteps < 1 || nsteps > 256) return fail(GP_ERR_INVALID, "gp_autotune: nsteps must be in [1, 256]");

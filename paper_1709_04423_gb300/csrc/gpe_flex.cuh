@@ -444,7 +444,10 @@ struct FlexPlan {
 // The tile is the widest of 16 lines and fewer that gives one and a half
 // blocks per SM.  Where the solving warps would still be fewer than four per SM
 // (an SM's FP64 rate needs four; the other chains only get shorter), free segments
-// are halved down to 8 points and FP64 and double-float take a thread per component.
+// are halved down to 8 points and FP64 and double-float take a thread per
+// component -- unless the line then needs more threads than a block has (over
+// 4098 points), which leaves both components to one thread: 5000 x 50 FP64
+// imaginary time 111 us per step, with a thread per line 8870.
 template <typename T>
 FlexPlan flex_plan(int n, long nlines, int seg, bool axis0, long reach) {
   FlexPlan p;
@@ -452,23 +455,25 @@ FlexPlan flex_plan(int n, long nlines, int seg, bool axis0, long reach) {
   const int lmin = axis0 ? 1 : sizeof(c2_t<T>) == 8 ? 2 : 1;
   const bool few = nlines * ((M + 15) / 16) < 32L * 4 * 152;
   p.split = few && !std::is_same<T, float>::value;
-  for (int lw = 4; lw >= 0; --lw) {
-    const int ls = lw + (p.split ? 1 : 0);
-    p.seg = seg;
-    if (seg == 0)
-      for (int sg : {8, 16, 32}) {
-        if (sg == 8 && !few) continue;
-        p.seg = sg;
-        if ((((M + sg - 1) / sg) << ls) <= kFlexMaxThreads) break;
-      }
-    p.t = flex_tile<T>(n, lw, p.seg);
-    p.t.depth = (int)std::max<long>(1, (reach + p.seg - 1) / p.seg);
-    p.threads = std::max(kFlexMinThreads, ((p.t.nseg << ls) + 31) / 32 * 32);
-    p.blocks = (unsigned)((nlines + (1L << lw) - 1) >> lw);
-    const bool fits = p.threads <= kFlexMaxThreads && flex_elems(p.t) * sizeof(c2_t<T>) <= 200 * 1024;
-    if (fits && (lw <= lmin || p.blocks >= 228)) return p;
+  for (;; p.split = false) {
+    for (int lw = 4; lw >= 0; --lw) {
+      const int ls = lw + (p.split ? 1 : 0);
+      p.seg = seg;
+      if (seg == 0)
+        for (int sg : {8, 16, 32}) {
+          if (sg == 8 && !few) continue;
+          p.seg = sg;
+          if ((((M + sg - 1) / sg) << ls) <= kFlexMaxThreads) break;
+        }
+      p.t = flex_tile<T>(n, lw, p.seg);
+      p.t.depth = (int)std::max<long>(1, (reach + p.seg - 1) / p.seg);
+      p.threads = std::max(kFlexMinThreads, ((p.t.nseg << ls) + 31) / 32 * 32);
+      p.blocks = (unsigned)((nlines + (1L << lw) - 1) >> lw);
+      const bool fits = p.threads <= kFlexMaxThreads && flex_elems(p.t) * sizeof(c2_t<T>) <= 200 * 1024;
+      if (fits && (lw <= lmin || p.blocks >= 228)) return p;
+    }
+    if (!p.split) return FlexPlan();
   }
-  return FlexPlan();
 }
 
 template <typename T, bool IMAG, bool LAST, int SEG, bool AXIS0, bool VAR, bool CLOSE>

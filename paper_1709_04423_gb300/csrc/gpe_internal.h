@@ -228,6 +228,24 @@ bool tma_x_fits(const gp_handle* h, int seg);  // the TMA x sweep takes this gri
 // kernel that fills it with NaN (all bits set) if the flag is set.  Only
 // handles that have launched a sweep with such waits (tma_used) need either.
 int fetch_dev_err(gp_handle* h);
+// the kernels a sweep may take (sweep_kind in gpe_step.cuh; gp_sweep_kernel's names)
+enum SweepKind {
+  SWEEP_LINE,    // 1d: every step of a run in one launch
+  SWEEP_NARROW,  // tiles of few lines
+  SWEEP_PLANE,   // the fused x + y sweeps
+  SWEEP_TMA,
+  SWEEP_PIPE,
+  SWEEP_TILE,    // x: 32-line shared-memory tiles
+  SWEEP_WARP,    // x: a warp per line
+  SWEEP_COLUMN,  // y/z: 32 lines per block
+  SWEEP_THREAD   // a thread per line
+};
+SweepKind sweep_kind_f32(const gp_handle* h, bool imag, int d);
+SweepKind sweep_kind_f64(const gp_handle* h, bool imag, int d);
+SweepKind sweep_kind_df(const gp_handle* h, bool imag, int d);
+bool takes_line_f32(const gp_handle* h);  // gp_step_* of this 1d grid runs in one launch
+bool takes_line_f64(const gp_handle* h);
+bool takes_line_df(const gp_handle* h);
 int take_dev_err(gp_handle* h, const char* who);
 // GP_ERR_CUDA (and clears it) if a sweep enqueued since the last call could not
 // be launched; the state is then not valid

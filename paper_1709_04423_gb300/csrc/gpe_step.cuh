@@ -430,6 +430,25 @@ FlexPlan flex_sweep(const gp_handle* h, bool imag, int d, int seg) {
   return flex_plan<T>(n, nlines, seg, d == 0, reach);
 }
 
+// The kernel that takes the sweep along axis d (from_src: the adjoint's x sweep,
+// which reads another buffer), with the plan of the tiles of few lines.
+template <typename T>
+SweepKind sweep_kind(const gp_handle* h, bool imag, int d, bool from_src, FlexPlan* plan) {
+  *plan = FlexPlan();
+  if (h->real_mode) return d == 0 ? SWEEP_TILE : SWEEP_COLUMN;
+  if (xy_fused(h) && !from_src && d < 2) return SWEEP_PLANE;
+  const int seg = d == 0 ? h->seg_x : h->seg_c;
+  *plan = flex_sweep<T>(h, imag, d, seg);
+  if (plan->threads > 0) return SWEEP_NARROW;
+  if (seg == 0) return SWEEP_THREAD;
+  if (h->geom != 2 || d > 0) {
+    if (std::is_same<T, float>::value && (d == 0 ? h->tma_x && !from_src : h->tma_c)) return SWEEP_TMA;
+    if (!is_df<T>::value && (d == 0 ? h->tile_x && h->pipe_x : h->pipe_c)) return SWEEP_PIPE;
+  }
+  if (d > 0) return SWEEP_COLUMN;
+  return h->tile_x ? SWEEP_TILE : SWEEP_WARP;
+}
+
 // Returns whether the sweep applied the step's closing N(dt/2).
 template <typename T>
 bool enqueue_sweep(gp_handle* h, bool imag, NormSlots ns, int d, const void* src = nullptr, bool half_open = true) {
@@ -442,16 +461,16 @@ bool enqueue_sweep(gp_handle* h, bool imag, NormSlots ns, int d, const void* src
   const double* parts_in = read ? h->parts[ns.rd] : nullptr;
   double* parts_out = write ? h->parts[ns.wr] : nullptr;
   unsigned blocks = 0;
-  const bool fuse_xy = xy_fused(h) && src == nullptr && (d == 0 || d == 1);
-  if (fuse_xy && d == 1) return false;  // done by the fused x + y kernel
-  const FlexPlan flex = flex_sweep<T>(h, imag, d, seg);
-  if (seg > 0 || flex.threads > 0) {
+  FlexPlan flex;
+  const SweepKind kind = sweep_kind<T>(h, imag, d, src != nullptr, &flex);
+  if (kind == SWEEP_PLANE && d == 1) return false;  // done by the fused x + y kernel
+  if (kind != SWEEP_THREAD) {
     Sweep2Args<T> a;
     std::memset(&a, 0, sizeof(a));
     a.psi = (c2_t<T>*)h->psi;
     a.src = d == 0 ? (const c2_t<T>*)src : nullptr;
     a.geom = geom_of(h, d);
-    const int si = seg_index(flex.threads > 0 ? flex.seg : seg);
+    const int si = seg_index(kind == SWEEP_NARROW ? flex.seg : seg);
     a.alpha = coef_ptr<T>(h, mode, d, 0);
     a.gf = coef_ptr<T>(h, mode, d, 1 + 2 * si);
     a.gb = coef_ptr<T>(h, mode, d, 2 + 2 * si);
@@ -476,7 +495,7 @@ bool enqueue_sweep(gp_handle* h, bool imag, NormSlots ns, int d, const void* src
       a.vh = cv + 2 * h->n[0];
     }
     bool done = false;
-    if (flex.threads > 0) {
+    if (kind == SWEEP_NARROW) {
       // Programmatic launches place a sweep's first blocks wherever the previous
       // one leaves room, so that some SMs take two of its one and a half blocks per
       // SM more than others: with the heavy blocks of long lines and of
@@ -495,7 +514,7 @@ bool enqueue_sweep(gp_handle* h, bool imag, NormSlots ns, int d, const void* src
       done = true;
     }
     if constexpr (std::is_same<T, float>::value) {
-      if (fuse_xy) {  // d == 0: the y axis' coefficients beside the x sweep's arguments
+      if (kind == SWEEP_PLANE) {  // d == 0: the y axis' coefficients beside the x sweep's arguments
         Sweep2Args<float> ay;
         std::memset(&ay, 0, sizeof(ay));
         ay.geom = geom_of(h, 1);
@@ -512,7 +531,7 @@ bool enqueue_sweep(gp_handle* h, bool imag, NormSlots ns, int d, const void* src
     }
     if (done) {
     } else if (var) {
-      if (h->tile_x) {  // axial trap: x is not the last axis
+      if (kind == SWEEP_TILE) {  // axial trap: x is not the last axis
         blocks = imag ? launch_t_seg<T, true, true, false, false, true>(seg, a, h->work, h->pdl_now)
                       : launch_t_seg<T, false, true, false, false, true>(seg, a, h->work, h->pdl_now);
       } else if (imag) {
@@ -524,14 +543,14 @@ bool enqueue_sweep(gp_handle* h, bool imag, NormSlots ns, int d, const void* src
       done = true;
     }
     if constexpr (std::is_same<T, float>::value) {
-      if (!done && d == 0 && h->tma_x && src == nullptr && !var) {
+      if (kind == SWEEP_TMA && d == 0) {
         blocks = seg == 8 ? (imag ? launch_tx<true, 8>(h, a, mode, h->work, h->pdl_now)
                                   : launch_tx<false, 8>(h, a, mode, h->work, h->pdl_now))
                           : (imag ? launch_tx<true, 16>(h, a, mode, h->work, h->pdl_now)
                                   : launch_tx<false, 16>(h, a, mode, h->work, h->pdl_now));
         done = true;
       }
-      if (!done && d > 0 && h->tma_c) {
+      if (kind == SWEEP_TMA && d > 0) {
         if (fuse_close) blocks = launch_tc_seg<true, true, true>(h, seg, a, h->work, h->pdl_now);
         else if (imag) blocks = write ? launch_tc_seg<true, true>(h, seg, a, h->work, h->pdl_now)
                                       : launch_tc_seg<true, false>(h, seg, a, h->work, h->pdl_now);
@@ -541,7 +560,7 @@ bool enqueue_sweep(gp_handle* h, bool imag, NormSlots ns, int d, const void* src
     }
     if constexpr (!is_df<T>::value) {  // pipelined shapes: FP32 and FP64 states only
       if (done) {
-      } else if (d == 0 && h->tile_x && h->pipe_x) {
+      } else if (kind == SWEEP_PIPE && d == 0) {
         if (imag) {
           blocks = write ? launch_p_seg<T, true, true, true, true>(seg, a, h->work, h->pdl_now)
                         : launch_p_seg<T, true, true, false, true>(seg, a, h->work, h->pdl_now);
@@ -549,7 +568,7 @@ bool enqueue_sweep(gp_handle* h, bool imag, NormSlots ns, int d, const void* src
           blocks = launch_p_seg<T, false, true, false, true>(seg, a, h->work, h->pdl_now);
         }
         done = true;
-      } else if (d > 0 && h->pipe_c) {
+      } else if (kind == SWEEP_PIPE) {
         if (imag) {
           blocks = write ? launch_p_seg<T, true, false, true, false>(seg, a, h->work, h->pdl_now)
                         : launch_p_seg<T, true, false, false, false>(seg, a, h->work, h->pdl_now);
@@ -560,14 +579,14 @@ bool enqueue_sweep(gp_handle* h, bool imag, NormSlots ns, int d, const void* src
       }
     }
     if (done) {
-    } else if (d == 0 && h->tile_x) {
+    } else if (kind == SWEEP_TILE) {
       if (imag) {
         blocks = write ? launch_t_seg<T, true, true, true>(seg, a, h->work, h->pdl_now)
                       : launch_t_seg<T, true, true, false>(seg, a, h->work, h->pdl_now);
       } else {
         blocks = launch_t_seg<T, false, true, false>(seg, a, h->work, h->pdl_now);
       }
-    } else if (d == 0) {
+    } else if (kind == SWEEP_WARP) {
       if (imag) {
         blocks = write ? launch_x_seg<T, true, true, true>(seg, a, h->work, h->pdl_now)
                       : launch_x_seg<T, true, true, false>(seg, a, h->work, h->pdl_now);

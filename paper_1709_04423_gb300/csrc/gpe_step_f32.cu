@@ -5,6 +5,11 @@ namespace gpe {
 
 int run_steps_f32(gp_handle* h, bool imag, long nsteps) { return run_steps_t<float>(h, imag, nsteps); }
 
+SweepKind sweep_kind_f32(const gp_handle* h, bool imag, int d) {
+  FlexPlan plan;
+  return sweep_kind<float>(h, imag, d, false, &plan);
+}
+
 int time_steps_f32(gp_handle* h, bool imag, long nsteps, double* ms_out) {
   return time_steps_t<float>(h, imag, nsteps, ms_out);
 }

@@ -46,6 +46,7 @@ ABI_SYMBOLS = (
     "gp_init_spherical", "gp_set_splitting", "gp_set_real_state", "gp_init_circular", "gp_init_axial",
     "gp_test_stall_transfers", "gp_time_sweeps_graph", "gp_fp_fma_rates", "gp_check_status",
     "gp_batch_set_mode", "gp_batch_get_mode", "gp_batch_autotune", "gp_test_batch_stall", "gp_test_refuse_maps",
+    "gp_sweep_kernel",
 )
 
 
@@ -105,6 +106,8 @@ def _open(path):
     lib.gp_time_sweeps_graph.argtypes = [_vp, I, I, ctypes.POINTER(D)]
     lib.gp_fp_fma_rates.argtypes = [ctypes.POINTER(D), ctypes.POINTER(D)]
     lib.gp_test_stall_transfers.argtypes = [_vp, I]
+    lib.gp_sweep_kernel.argtypes = [_vp, I, I]
+    lib.gp_sweep_kernel.restype = ctypes.c_char_p
     lib.gp_test_refuse_maps.argtypes = [_vp, I]
     lib.gp_check_status.argtypes = [ctypes.POINTER(I)]
     lib.gp_observables_noalloc.argtypes = [I, ctypes.POINTER(I), ctypes.POINTER(D), ctypes.POINTER(D), D, I,
@@ -290,6 +293,12 @@ def gp_get_shapes(h):
     t, x, c, k = ctypes.c_int(), ctypes.c_int(), ctypes.c_int(), ctypes.c_int()
     _check(load().gp_get_shapes(h, ctypes.byref(t), ctypes.byref(x), ctypes.byref(c), ctypes.byref(k)))
     return {"tile_x": t.value, "seg_x": x.value, "seg_c": c.value, "flags": k.value}
+
+
+def gp_sweep_kernel(h, imag, axis):
+    """Name of the kernel that takes the sweep along an axis (None: no such sweep)."""
+    name = load().gp_sweep_kernel(h, int(bool(imag)), int(axis))
+    return name.decode() if name else None
 
 
 def gp_adjoint_forward(h, nsteps, ckpt_every):
@@ -520,6 +529,10 @@ class Propagator:
 
     def shapes(self):
         return gp_get_shapes(self.h)
+
+    def sweep_kernels(self, imag):
+        """The kernels that take the sweeps along x, y, z (see gp_sweep_kernel)."""
+        return [gp_sweep_kernel(self.h, imag, d) for d in range(self.dim)]
 
     def autotune(self, imag, nsteps=8, cache=True):
         """Picks the fastest kernel shapes for this grid (see gp_autotune).
