@@ -141,6 +141,7 @@ struct gp_handle {
   double* parts[2] = {nullptr, nullptr};
   int parts_n = 0;
   double parts_ws = 1.0;
+  bool norm_folded = false;  // the last sweep's sums are folded into one (a launch of its own)
   bool pdl_now = false;
   double* red_parts = nullptr;  // reduced-density chunk sums (+ host-bound output)
   size_t red_cap = 0;
