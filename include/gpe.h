@@ -380,8 +380,18 @@ int gp_observables_noalloc(int dim, const int n[3], const double dx[3], const do
  * y/z input segment is kept in registers or streamed and read again, and
  * whether the x and y/z sweeps run as persistent double-buffered kernels
  * (possible where two 32-line tiles fit in shared memory); shape 0 means the
- * general kernels used for lines longer than 514 points.  Defaults are set by
- * gp_init.  gp_autotune times every valid shape of the x sweep and of the y/z
+ * general kernels used for lines longer than 514 points (tiles of few lines,
+ * 1d: every step of a run in one launch; a thread per line where a line is too
+ * long for those).  Defaults are set by gp_init; gp_sweep_kernel names the
+ * kernel that a sweep takes.
+ * GP_SHAPE_NARROW_X / GP_SHAPE_NARROW_YZ (the default where they apply): a
+ * sweep whose grid has few 32-line tiles runs on tiles of 1 to 16 lines, and
+ * the x lines that no 32-line tile holds do; on 1d grids GP_SHAPE_NARROW_X
+ * runs every step of a call in one launch.  The segment length is the handle's
+ * on Cartesian grids in real time and in 3d, else free.  gp_set_shapes drops
+ * the flags where no sweep of the grid takes them; the pipelined, fused and
+ * TMA forms of a sweep come before them.
+ * gp_autotune times every valid shape of the x sweep and of the y/z
  * sweeps on this handle's grid (2 warm-up + nsteps timed steps each, imaginary
  * time if imag != 0; 1 <= nsteps <= 256), keeps the fastest, restores the
  * state, and remembers the result for this process (a later call for the same
@@ -413,7 +423,9 @@ enum {
   GP_SHAPE_PIPE_YZ = 4, /* y/z sweeps: persistent double-buffered kernel */
   GP_SHAPE_FUSE_XY = 8, /* x and y sweeps fused, one block per xy plane (3d FP32) */
   GP_SHAPE_TMA_YZ = 16, /* y/z sweeps: persistent kernel, tiles moved by TMA (FP32) */
-  GP_SHAPE_TMA_X = 32   /* x sweep (with N): persistent kernel, tiles moved by TMA (FP32) */
+  GP_SHAPE_TMA_X = 32,  /* x sweep (with N): persistent kernel, tiles moved by TMA (FP32) */
+  GP_SHAPE_NARROW_X = 64,  /* x sweep: tiles of few lines where there are few; 1d: a run in one launch */
+  GP_SHAPE_NARROW_YZ = 128 /* y/z sweeps: tiles of few lines where there are few */
 };
 int gp_autotune(gp_handle* h, int imag, int nsteps, double* best_ms);
 int gp_set_shapes(gp_handle* h, int tile_x, int seg_x, int seg_c, int flags);

@@ -479,6 +479,31 @@ int tile_seg(int M) {
 
 namespace {
 
+bool takes_line(const gp_handle* h) {
+  return h->prec == GP_DF64 ? takes_line_df(h) : h->prec == GP_F64 ? takes_line_f64(h) : takes_line_f32(h);
+}
+
+// Whether gp_step_* of this 1d grid runs in one launch (gpe_line.cuh).
+bool line_run(const gp_handle* h) { return h->dim == 1 && (h->seg_x == 0 || h->narrow_x) && takes_line(h); }
+
+// Sets narrow_x and narrow_c where wanted and where a sweep of the grid takes
+// them, so that gp_get_shapes reports what runs (a real state's sweeps never
+// do; its complex state keeps its flags).
+void set_narrow(gp_handle* h, bool x, bool c) {
+  if (h->real_mode) return;
+  h->narrow_x = x && h->seg_x > 0;
+  h->narrow_c = c && h->dim > 1 && h->seg_c > 0;
+  if (h->dim == 1) {
+    h->narrow_x = h->narrow_x && takes_line(h);
+    return;
+  }
+  auto taken = [&](int d) {
+    return sweep_kind_any(h, true, d) == SWEEP_NARROW || sweep_kind_any(h, false, d) == SWEEP_NARROW;
+  };
+  h->narrow_x = h->narrow_x && taken(0);
+  h->narrow_c = h->narrow_c && (taken(1) || (h->dim > 2 && taken(2)));
+}
+
 // Defaults of 3d Cartesian grids, where the autotuner's picks agree over many
 // sizes (us per sweep of the x, y, z sweeps, the general rule's shape -> this one):
 //  * FP64 is bound by its FP64 pipe: longer segments carry less (128^3 real
@@ -548,6 +573,7 @@ void choose_shapes(gp_handle* h) {
   for (const char* e : {"GPE_TILE_X", "GPE_SEG_X", "GPE_SEG_YZ", "GPE_KEEP", "GPE_PIPE", "GPE_FUSE_XY"})
     forced = forced || std::getenv(e);
   if (h->dim == 3 && h->geom == 0 && !forced) choose_shapes_3d(h);
+  set_narrow(h, !forced, !forced);
 }
 
 }  // namespace
@@ -557,18 +583,58 @@ int upload_coefs(gp_handle* h) {
   return h->prec == GP_F64 ? upload_coefs_t<double>(h) : upload_coefs_t<float>(h);
 }
 
+SweepKind sweep_kind_any(const gp_handle* h, bool imag, int d, int* plan) {
+  int unused = 0;
+  if (!plan) plan = &unused;
+  return h->prec == GP_DF64  ? sweep_kind_df(h, imag, d, plan)
+         : h->prec == GP_F64 ? sweep_kind_f64(h, imag, d, plan)
+                             : sweep_kind_f32(h, imag, d, plan);
+}
+
+namespace {
+
+// nsteps > 0 steps of a 1d grid in one launch
+int run_line_any(gp_handle* h, bool imag, long nsteps) {
+  return h->prec == GP_DF64  ? run_line_df(h, imag, nsteps)
+         : h->prec == GP_F64 ? run_line_f64(h, imag, nsteps)
+                             : run_line_f32(h, imag, nsteps);
+}
+
+// The time per step of such a run (events on the library's stream), as the x sweep's
+int time_line(gp_handle* h, bool imag, long nsteps, double* ms_out) {
+  ms_out[0] = ms_out[1] = ms_out[2] = 0.0;
+  if (nsteps == 0) return GP_OK;
+  cudaEvent_t ev[2] = {nullptr, nullptr};
+  int rc = join_in(h);
+  if (rc) return rc;
+  cudaError_t e = cudaEventCreate(&ev[0]);
+  if (e == cudaSuccess) e = cudaEventCreate(&ev[1]);
+  if (e == cudaSuccess) e = cudaEventRecord(ev[0], h->work);
+  if (e == cudaSuccess) rc = run_line_any(h, imag, nsteps);
+  if (e == cudaSuccess && !rc) e = cudaEventRecord(ev[1], h->work);
+  if (e == cudaSuccess && !rc) e = cudaEventSynchronize(ev[1]);
+  float ms = 0.f;
+  if (e == cudaSuccess && !rc) e = cudaEventElapsedTime(&ms, ev[0], ev[1]);
+  for (auto& x : ev)
+    if (x) cudaEventDestroy(x);
+  if (!rc && e != cudaSuccess) rc = fail(GP_ERR_CUDA, std::string("gp_time_sweeps: ") + cudaGetErrorString(e));
+  ms_out[0] = ms / nsteps;
+  return rc;
+}
+
+}  // namespace
+
 // Step launchers of the handle's state precision.
 int run_steps_any(gp_handle* h, bool imag, long nsteps) {
-  if (h->dim == 1 && nsteps > 0) {
-    const int rc = h->prec == GP_DF64  ? run_line_df(h, imag, nsteps)
-                   : h->prec == GP_F64 ? run_line_f64(h, imag, nsteps)
-                                       : run_line_f32(h, imag, nsteps);
+  if (nsteps > 0 && line_run(h)) {
+    const int rc = run_line_any(h, imag, nsteps);
     if (rc != GP_ERR_STATE) return rc;
   }
   if (h->prec == GP_DF64) return run_steps_df(h, imag, nsteps);
   return h->prec == GP_F64 ? run_steps_f64(h, imag, nsteps) : run_steps_f32(h, imag, nsteps);
 }
 int time_steps_any(gp_handle* h, bool imag, long nsteps, double* ms) {
+  if (line_run(h)) return time_line(h, imag, nsteps, ms);
   if (h->prec == GP_DF64) return time_steps_df(h, imag, nsteps, ms);
   return h->prec == GP_F64 ? time_steps_f64(h, imag, nsteps, ms) : time_steps_f32(h, imag, nsteps, ms);
 }
@@ -1058,7 +1124,8 @@ int gp_time_sweeps_graph(gp_handle* h, int imag, int reps, double* ms_per_launch
     if (e != cudaSuccess) rc = fail(GP_ERR_CUDA, cudaGetErrorString(e));
   }
   if (!rc) {
-    rc = h->prec == GP_DF64 ? time_graph_df(h, imag != 0, reps, ms_per_launch)
+    rc = line_run(h)          ? time_line(h, imag != 0, reps, ms_per_launch)
+         : h->prec == GP_DF64 ? time_graph_df(h, imag != 0, reps, ms_per_launch)
          : h->prec == GP_F64 ? time_graph_f64(h, imag != 0, reps, ms_per_launch)
                              : time_graph_f32(h, imag != 0, reps, ms_per_launch);
   }
@@ -1290,6 +1357,7 @@ int gp_set_shapes(gp_handle* h, int tile_x, int seg_x, int seg_c, int flags) {
   h->pipe_x = px;
   h->pipe_c = pc;
   h->xyfuse = fxy;
+  set_narrow(h, (flags & GP_SHAPE_NARROW_X) != 0, (flags & GP_SHAPE_NARROW_YZ) != 0);
   return GP_OK;
 }
 
@@ -1301,20 +1369,14 @@ int gp_get_shapes(const gp_handle* h, int* tile_x, int* seg_x, int* seg_c, int* 
   if (flags)
     *flags = (h->keep_c ? GP_SHAPE_KEEP_YZ : 0) | (h->pipe_x ? GP_SHAPE_PIPE_X : 0) |
              (h->pipe_c ? GP_SHAPE_PIPE_YZ : 0) | (h->xyfuse ? GP_SHAPE_FUSE_XY : 0) |
-             (h->tma_c ? GP_SHAPE_TMA_YZ : 0) | (h->tma_x ? GP_SHAPE_TMA_X : 0);
+             (h->tma_c ? GP_SHAPE_TMA_YZ : 0) | (h->tma_x ? GP_SHAPE_TMA_X : 0) |
+             (h->narrow_x ? GP_SHAPE_NARROW_X : 0) | (h->narrow_c ? GP_SHAPE_NARROW_YZ : 0);
   return GP_OK;
 }
 
 const char* gp_sweep_kernel(const gp_handle* h, int imag, int axis) {
   if (!h || axis < 0 || axis >= h->dim || (h->real_mode && !imag)) return nullptr;
-  SweepKind k;
-  if (h->dim == 1 && (h->prec == GP_DF64 ? takes_line_df(h) : h->prec == GP_F64 ? takes_line_f64(h) : takes_line_f32(h)))
-    k = SWEEP_LINE;
-  else
-    k = h->prec == GP_DF64  ? sweep_kind_df(h, imag != 0, axis)
-        : h->prec == GP_F64 ? sweep_kind_f64(h, imag != 0, axis)
-                            : sweep_kind_f32(h, imag != 0, axis);
-  switch (k) {
+  switch (line_run(h) ? SWEEP_LINE : sweep_kind_any(h, imag != 0, axis)) {
     case SWEEP_LINE: return "line";
     case SWEEP_NARROW: return "narrow";
     case SWEEP_PLANE: return "plane";
@@ -1341,30 +1403,69 @@ int gp_autotune(gp_handle* h, int imag, int nsteps, double* best_ms) {
     }
   }
   // candidate shapes for the x sweep and for the y/z sweeps (timed separately)
-  std::vector<std::array<int, 4>> xs;  // (tile, seg, pipelined, TMA)
+  std::vector<std::array<int, 5>> xs;  // (tile, seg, pipelined, TMA, narrow)
   for (int sg : {4, 8, 16, 32})
     if (shapes_valid(h, 1, sg, h->seg_c)) {
-      xs.push_back({1, sg, 0, 0});
-      if (h->prec != GP_DF64 && !real && h->geom != 2 && pipe_fits(h, h->n[0], true)) xs.push_back({1, sg, 1, 0});
-      if (!real && tma_x_fits(h, sg)) xs.push_back({1, sg, 0, 1});
+      xs.push_back({1, sg, 0, 0, 0});
+      if (h->prec != GP_DF64 && !real && h->geom != 2 && pipe_fits(h, h->n[0], true)) xs.push_back({1, sg, 1, 0, 0});
+      if (!real && tma_x_fits(h, sg)) xs.push_back({1, sg, 0, 1, 0});
     }
+  const bool x_tiles = !xs.empty();
   for (int sg : {1, 2, 4, 8, 16})
-    if (!real && shapes_valid(h, 0, sg, h->seg_c)) { xs.push_back({0, sg, 0, 0}); break; }
-  std::vector<std::array<int, 4>> cs;  // (seg, keep input in registers, pipelined, TMA)
+    if (!real && shapes_valid(h, 0, sg, h->seg_c)) { xs.push_back({0, sg, 0, 0, 0}); break; }
+  std::vector<std::array<int, 5>> cs;  // (seg, keep input in registers, pipelined, TMA, narrow)
   int nmax = 0;
   for (int d = 1; d < h->dim; ++d) nmax = std::max(nmax, h->n[d]);
   if (h->dim > 1)
     for (int sg : {4, 8, 16, 32})
       if (shapes_valid(h, h->tile_x, h->seg_x, sg)) {
-        if (sg * (int)h->esize / 2 <= 64) cs.push_back({sg, 1, 0, 0});
-        cs.push_back({sg, 0, 0, 0});
-        if (h->prec != GP_DF64 && !real && pipe_fits(h, nmax, false)) cs.push_back({sg, 0, 1, 0});
-        if (!real && tma_fits(h, sg)) cs.push_back({sg, 0, 0, 1});
+        if (sg * (int)h->esize / 2 <= 64) cs.push_back({sg, 1, 0, 0, 0});
+        cs.push_back({sg, 0, 0, 0, 0});
+        if (h->prec != GP_DF64 && !real && pipe_fits(h, nmax, false)) cs.push_back({sg, 0, 1, 0, 0});
+        if (!real && tma_fits(h, sg)) cs.push_back({sg, 0, 0, 1, 0});
       }
   const int keep_t = h->tile_x, keep_x = h->seg_x, keep_c = h->seg_c, keep_k = h->keep_c;
   const bool keep_px = h->pipe_x, keep_pc = h->pipe_c, keep_fxy = h->xyfuse, keep_tc = h->tma_c;
-  const bool keep_tx = h->tma_x;
+  const bool keep_tx = h->tma_x, keep_nx = h->narrow_x, keep_nc = h->narrow_c;
   h->xyfuse = false;  // the separate sweeps first
+  auto apply = [&](int t, int sx, int px, int tx, int nx, int sc, int kc, int pc, int tc, int nc) {
+    h->tile_x = t != 0;
+    h->seg_x = sx;
+    h->pipe_x = px != 0;
+    h->tma_x = tx != 0;
+    h->narrow_x = nx != 0;
+    h->seg_c = sc;
+    h->keep_c = kc;
+    h->pipe_c = pc != 0;
+    h->tma_c = tc != 0;
+    h->narrow_c = nc != 0;
+  };
+  // tiles of few lines: each plan once (several segment lengths can lead to the same)
+  if (!real) {
+    std::vector<std::array<int, 2>> seen;
+    auto is_new = [&](int d0, int d1) {
+      std::array<int, 2> id = {0, 0};
+      for (int d = d0; d < d1; ++d) {
+        int plan = 0;
+        if (sweep_kind_any(h, imag != 0, d, &plan) == SWEEP_NARROW) id[d - d0] = plan + 1;
+      }
+      if ((id[0] == 0 && id[1] == 0) || std::find(seen.begin(), seen.end(), id) != seen.end()) return false;
+      seen.push_back(id);
+      return true;
+    };
+    for (const auto& c : std::vector<std::array<int, 5>>(xs)) {
+      if (c[2] || c[3] || (c[0] == 0 && x_tiles)) continue;
+      apply(c[0], c[1], 0, 0, 1, keep_c, keep_k, keep_pc, keep_tc, keep_nc);
+      if (h->dim == 1 ? takes_line(h) : is_new(0, 1)) xs.push_back({c[0], c[1], 0, 0, 1});
+    }
+    seen.clear();
+    for (const auto& c : std::vector<std::array<int, 5>>(cs)) {
+      if (c[1] || c[2] || c[3]) continue;
+      apply(keep_t, keep_x, keep_px, keep_tx, keep_nx, c[0], 0, 0, 0, 1);
+      if (is_new(1, h->dim)) cs.push_back({c[0], 0, 0, 0, 1});
+    }
+    apply(keep_t, keep_x, keep_px, keep_tx, keep_nx, keep_c, keep_k, keep_pc, keep_tc, keep_nc);
+  }
   void* saved = nullptr;
   void* const state = real ? h->rpsi : h->psi;
   const size_t sbytes = (size_t)h->np * (real ? h->esize / 2 : h->esize);
@@ -1374,15 +1475,9 @@ int gp_autotune(gp_handle* h, int imag, int nsteps, double* best_ms) {
     cudaError_t e = cudaMemcpyAsync(saved, state, sbytes, cudaMemcpyDeviceToDevice, h->work);
     if (e != cudaSuccess) rc = fail(GP_ERR_CUDA, cudaGetErrorString(e));
   }
-  auto time_shape = [&](int t, int sx, int px, int tx, int sc, int kc, int pc, int tc, double* ms3) -> int {
-    h->tile_x = t != 0;
-    h->seg_x = sx;
-    h->pipe_x = px != 0;
-    h->tma_x = tx != 0;
-    h->seg_c = sc;
-    h->keep_c = kc;
-    h->pipe_c = pc != 0;
-    h->tma_c = tc != 0;
+  auto time_shape = [&](int t, int sx, int px, int tx, int nx, int sc, int kc, int pc, int tc, int nc,
+                        double* ms3) -> int {
+    apply(t, sx, px, tx, nx, sc, kc, pc, tc, nc);
     double warm[3];
     int r = time_steps_any(h, imag != 0, 2, warm);
     if (r) return r;
@@ -1390,19 +1485,19 @@ int gp_autotune(gp_handle* h, int imag, int nsteps, double* best_ms) {
   };
   double bx = 1e30, bc = 1e30;
   int best_t = keep_t, best_x = keep_x, best_c = keep_c, best_k = keep_k, best_px = keep_px, best_pc = keep_pc;
-  int best_tc = keep_tc, best_tx = keep_tx;
+  int best_tc = keep_tc, best_tx = keep_tx, best_nx = keep_nx, best_nc = keep_nc;
   for (const auto& c : xs) {
     if (rc) break;
     double ms[3];
-    rc = time_shape(c[0], c[1], c[2], c[3], keep_c, keep_k, keep_pc, keep_tc, ms);
-    if (!rc && ms[0] < bx) { bx = ms[0]; best_t = c[0]; best_x = c[1]; best_px = c[2]; best_tx = c[3]; }
+    rc = time_shape(c[0], c[1], c[2], c[3], c[4], keep_c, keep_k, keep_pc, keep_tc, keep_nc, ms);
+    if (!rc && ms[0] < bx) { bx = ms[0]; best_t = c[0]; best_x = c[1]; best_px = c[2]; best_tx = c[3]; best_nx = c[4]; }
   }
   for (const auto& c : cs) {
     if (rc) break;
     double ms[3];
-    rc = time_shape(best_t, best_x, best_px, best_tx, c[0], c[1], c[2], c[3], ms);
+    rc = time_shape(best_t, best_x, best_px, best_tx, best_nx, c[0], c[1], c[2], c[3], c[4], ms);
     const double t = ms[1] + ms[2];
-    if (!rc && t < bc) { bc = t; best_c = c[0]; best_k = c[1]; best_pc = c[2]; best_tc = c[3]; }
+    if (!rc && t < bc) { bc = t; best_c = c[0]; best_k = c[1]; best_pc = c[2]; best_tc = c[3]; best_nc = c[4]; }
   }
   // the fused x + y sweeps, with the best z shape, against the best separate ones
   // (8- and 16-point segments: 32-point ones spill under the 64 registers a
@@ -1413,7 +1508,7 @@ int gp_autotune(gp_handle* h, int imag, int nsteps, double* best_ms) {
       if (rc || !plane_fits(h, sg) || !shapes_valid(h, 1, sg, best_c)) continue;
       double ms[3];
       h->xyfuse = true;
-      rc = time_shape(1, sg, 0, 0, best_c, best_k, best_pc, best_tc, ms);
+      rc = time_shape(1, sg, 0, 0, 0, best_c, best_k, best_pc, best_tc, best_nc, ms);
       h->xyfuse = false;
       if (!rc && ms[0] + ms[1] + ms[2] < bx + bc) {
         bx = ms[0] + ms[1];
@@ -1423,6 +1518,7 @@ int gp_autotune(gp_handle* h, int imag, int nsteps, double* best_ms) {
         best_x = sg;
         best_px = 0;
         best_tx = 0;
+        best_nx = 0;
       }
     }
   if (!rc) {
@@ -1433,10 +1529,11 @@ int gp_autotune(gp_handle* h, int imag, int nsteps, double* best_ms) {
   cudaFree(saved);
   const int best_flags = (best_k ? GP_SHAPE_KEEP_YZ : 0) | (best_px ? GP_SHAPE_PIPE_X : 0) |
                          (best_pc ? GP_SHAPE_PIPE_YZ : 0) | (best_fxy ? GP_SHAPE_FUSE_XY : 0) |
-                         (best_tc ? GP_SHAPE_TMA_YZ : 0) | (best_tx ? GP_SHAPE_TMA_X : 0);
+                         (best_tc ? GP_SHAPE_TMA_YZ : 0) | (best_tx ? GP_SHAPE_TMA_X : 0) |
+                         (best_nx ? GP_SHAPE_NARROW_X : 0) | (best_nc ? GP_SHAPE_NARROW_YZ : 0);
+  if (rc || real) apply(keep_t, keep_x, keep_px, keep_tx, keep_nx, keep_c, keep_k, keep_pc, keep_tc, keep_nc);
   if (rc) {
-    h->tile_x = keep_t; h->seg_x = keep_x; h->seg_c = keep_c; h->keep_c = keep_k;
-    h->pipe_x = keep_px; h->pipe_c = keep_pc; h->xyfuse = keep_fxy; h->tma_c = keep_tc; h->tma_x = keep_tx;
+    h->xyfuse = keep_fxy;
     return rc;
   }
   {

@@ -121,6 +121,9 @@ struct gp_handle {
   // 514 points: gpe_flex.cuh, else the thread-per-line kernel) and whether the x lines are staged through a shared-memory tile
   int seg_x = 0, seg_c = 0;
   bool tile_x = false;
+  // tiles of few lines where the grid has few 32-line ones (flex_sweep); 1d: a
+  // whole run in one launch (set_narrow)
+  bool narrow_x = false, narrow_c = false;
   int keep_c = 1;  // y/z sweeps keep their input segment in registers (when short enough)
   // persistent double-buffered sweeps (x needs tile_x); only where two
   // shared-memory stages of 32 lines fit
@@ -241,10 +244,12 @@ enum SweepKind {
   SWEEP_COLUMN,  // y/z: 32 lines per block
   SWEEP_THREAD   // a thread per line
 };
-SweepKind sweep_kind_f32(const gp_handle* h, bool imag, int d);
-SweepKind sweep_kind_f64(const gp_handle* h, bool imag, int d);
-SweepKind sweep_kind_df(const gp_handle* h, bool imag, int d);
-bool takes_line_f32(const gp_handle* h);  // gp_step_* of this 1d grid runs in one launch
+// plan: SWEEP_NARROW's tile width and segment length, in one number
+SweepKind sweep_kind_f32(const gp_handle* h, bool imag, int d, int* plan);
+SweepKind sweep_kind_f64(const gp_handle* h, bool imag, int d, int* plan);
+SweepKind sweep_kind_df(const gp_handle* h, bool imag, int d, int* plan);
+SweepKind sweep_kind_any(const gp_handle* h, bool imag, int d, int* plan = nullptr);
+bool takes_line_f32(const gp_handle* h);  // the one-launch kernel can hold this 1d grid's line
 bool takes_line_f64(const gp_handle* h);
 bool takes_line_df(const gp_handle* h);
 int take_dev_err(gp_handle* h, const char* who);

@@ -392,6 +392,8 @@ inline bool strang_close_fused(const gp_handle* h, bool imag) {
 
 // The tiles of few lines (gpe_flex.cuh) of the sweep along axis d, or threads =
 // 0 where another kernel takes it.  They take lines of more than 514 points
+// and, where the handle's shapes have them (narrow_x, narrow_c: the default),
+// the grids named below
 // (without them a thread walks a whole line: 1000 x 1000 FP64 imaginary time
 // 2840 -> 150 us per step), x lines for which no 32-line tile was chosen, and
 // grids with few 32-line tiles (us per sweep, 32-line tiles -> these):
@@ -417,6 +419,7 @@ FlexPlan flex_sweep(const gp_handle* h, bool imag, int d, int seg) {
   if (h->dim == 1 || h->real_mode) return FlexPlan();
   const long reach = h->axis_reach[imag ? MODE_IMAG : MODE_REAL][d];
   if (seg > 0) {
+    if (!(d == 0 ? h->narrow_x : h->narrow_c)) return FlexPlan();
     if (d == 0 ? h->pipe_x || h->tma_x : h->pipe_c || h->tma_c) return FlexPlan();
     if (d < 2 && xy_fused(h)) return FlexPlan();
     if (d == 0 && !h->tile_x) seg = tile_seg(n - 2);

@@ -61,9 +61,11 @@ void tf_from_c128(gp_handle* h, void* dst, const void* src, long n) {
 
 int run_steps_df(gp_handle* h, bool imag, long nsteps) { return run_steps_t<df64>(h, imag, nsteps); }
 
-SweepKind sweep_kind_df(const gp_handle* h, bool imag, int d) {
-  FlexPlan plan;
-  return sweep_kind<df64>(h, imag, d, false, &plan);
+SweepKind sweep_kind_df(const gp_handle* h, bool imag, int d, int* plan) {
+  FlexPlan p;
+  const SweepKind k = sweep_kind<df64>(h, imag, d, false, &p);
+  *plan = p.seg * 8 + p.t.lw;
+  return k;
 }
 
 int time_steps_df(gp_handle* h, bool imag, long nsteps, double* ms_out) {

@@ -5,9 +5,11 @@ namespace gpe {
 
 int run_steps_f64(gp_handle* h, bool imag, long nsteps) { return run_steps_t<double>(h, imag, nsteps); }
 
-SweepKind sweep_kind_f64(const gp_handle* h, bool imag, int d) {
-  FlexPlan plan;
-  return sweep_kind<double>(h, imag, d, false, &plan);
+SweepKind sweep_kind_f64(const gp_handle* h, bool imag, int d, int* plan) {
+  FlexPlan p;
+  const SweepKind k = sweep_kind<double>(h, imag, d, false, &p);
+  *plan = p.seg * 8 + p.t.lw;
+  return k;
 }
 
 int time_steps_f64(gp_handle* h, bool imag, long nsteps, double* ms_out) {

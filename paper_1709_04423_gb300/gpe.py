@@ -33,6 +33,8 @@ GP_SHAPE_PIPE_X = 2
 GP_SHAPE_PIPE_YZ = 4
 GP_SHAPE_TMA_YZ = 16
 GP_SHAPE_TMA_X = 32
+GP_SHAPE_NARROW_X = 64
+GP_SHAPE_NARROW_YZ = 128
 GP_SHAPE_FUSE_XY = 8
 
 # every entry point declared in include/gpe.h
@@ -543,7 +545,8 @@ class Propagator:
         import torch
         path = os.environ.get("GPE_TUNE_CACHE", os.path.join(os.path.expanduser("~"), ".cache", "gpe_gb300",
                                                              "shapes.json"))
-        key = "|".join([torch.cuda.get_device_name(), "x".join(map(str, self.n)), self.precision,
+        # (the leading "narrow": entries made before the tiles of few lines were a shape lack their flags)
+        key = "|".join(["narrow", torch.cuda.get_device_name(), "x".join(map(str, self.n)), self.precision,
                         "imag" if imag else "real"] + (["real_state"] if self.real_state else []))
         table = {}
         if cache and os.path.exists(path):
