@@ -386,7 +386,7 @@ int gp_observables_noalloc(int dim, const int n[3], const double dx[3], const do
  * kernel that a sweep takes.
  * GP_SHAPE_NARROW_X / GP_SHAPE_NARROW_YZ (the default where they apply): a
  * sweep whose grid has few 32-line tiles runs on tiles of 1 to 16 lines, and
- * the x lines that no 32-line tile holds do; on 1d grids GP_SHAPE_NARROW_X
+ * so does the x sweep of any grid without the x tile; on 1d grids GP_SHAPE_NARROW_X
  * runs every step of a call in one launch.  The segment length is the handle's
  * on Cartesian grids in real time and in 3d, else free.  gp_set_shapes drops
  * the flags where no sweep of the grid takes them; the pipelined, fused and
