@@ -472,8 +472,40 @@ LinePlan line_plan(int M) {
   return p;
 }
 
+// Whether the current device can hold a cluster of C blocks of this kernel
+// (up to 8 blocks every device can; 16 depend on the device and the block's
+// size, and are an attribute of the kernel that each device's context keeps).
+template <typename T, bool IMAG, bool VAR, int S>
+bool line_fits(int C, int threads) {
+  if (C <= 8) return true;
+  constexpr int kDevices = 64;
+  static std::atomic<signed char> known[kDevices][kLineMaxThreads / 32 + 1] = {};  // 0: not asked; 1: yes; 2: no
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kDevices) return false;
+  auto& k = known[dev][threads / 32];
+  if (k.load() == 0) {
+    auto kern = line_steps_kernel<T, IMAG, VAR, S>;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(C);
+    cfg.blockDim = dim3(threads);
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = C;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    int clusters = 0;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg);
+    if (e != cudaSuccess) cudaGetLastError();
+    k.store(e == cudaSuccess && clusters > 0 ? 1 : 2);
+  }
+  return k.load() == 1;
+}
+
 template <typename T, bool IMAG, bool VAR, int S>
 int launch_line(gp_handle* h, const LineArgs<T>& a, int C, int threads) {
+  if (!line_fits<T, IMAG, VAR, S>(C, threads)) return GP_ERR_STATE;
   auto kern = line_steps_kernel<T, IMAG, VAR, S>;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(C);
@@ -485,17 +517,6 @@ int launch_line(gp_handle* h, const LineArgs<T>& a, int C, int threads) {
   at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = C > 1 ? 1 : 0;
-  if (C > 8) {  // beyond the portable cluster size: only where the device can hold such a cluster
-    static std::atomic<int> fits{-1};
-    if (fits.load() < 0) {
-      int clusters = 0;
-      cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-      if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg);
-      if (e != cudaSuccess) cudaGetLastError();
-      fits.store(e == cudaSuccess && clusters > 0 ? 1 : 0);
-    }
-    if (!fits.load()) return GP_ERR_STATE;
-  }
   GP_CUDA(cudaLaunchKernelEx(&cfg, kern, a));
   count_launch();
   return GP_OK;
