@@ -79,9 +79,9 @@ __device__ __forceinline__ void st_cluster(V* dst, unsigned rank, V v) {
                  : "memory");
 }
 
-// 1/sqrt(s): the FP32 estimate and one third-order Newton correction, y = y0 (1
-// + r/2 + 3 r^2/8) with r = 1 - s y0^2 about 2^-22 (the omitted term is below
-// 2^-66); outside the FP32 range the library functions.
+// 1/sqrt(s) = y0 (1 - r)^(-1/2) with the FP32 estimate y0 and r = 1 - s y0^2,
+// about 2^-22: the binomial series to second order, y0 (1 + r/2 + 3 r^2/8) (the
+// omitted term is below 2^-66); outside the FP32 range the library functions.
 __device__ __forceinline__ double line_rsqrt(double s) {
   if (!(s > 1e-30 && s < 1e30)) return 1.0 / ::sqrt(s);
   const double y0 = (double)rsqrtf((float)s);
