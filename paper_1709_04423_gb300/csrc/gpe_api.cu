@@ -507,13 +507,20 @@ void set_narrow(gp_handle* h, bool x, bool c) {
 // Defaults of 3d Cartesian grids, where the autotuner's picks agree over many
 // sizes (us per sweep of the x, y, z sweeps, the general rule's shape -> this one):
 //  * FP64 is bound by its FP64 pipe: longer segments carry less (128^3 real
-//    time 218 / 116 / 116 -> 196 / 92 / 92, 96^3 83 / 44 / 44 -> 76 / 38 / 38),
-//    unless a short axis leaves them partly empty (z of 90 points in segments of
-//    16: 53 -> 65);
-//  * FP32 states that do not stay in L2 between sweeps stream through the TMA
-//    sweeps (256^3 real 92 / 70 / 73 -> 59 / 48 / 49, 160 x 144 x 150 imaginary
-//    24 / 16 / 18 -> 18 / 11 / 15); those that do and whose xy planes nearly fill
-//    the SMs take the fused x + y sweep (128^3 imaginary 16.1 + 7.8 -> 18.4).
+//    time 218 / 116 / 116 -> 196 / 92 / 92, 96^3 83 / 44 / 44 -> 76 / 38 / 38).
+//    y and z share one segment length, and the last wave of blocks decides which
+//    is better for the shorter of them, so the line of 90 points is that of one
+//    grid: 120 x 101 x 90, z in segments of 8 53, of 16 65.  (96 x 96 x nz gains
+//    from 16 at any nz: 64 points 28.4 -> 26.9, 80 37.9 -> 32.7, 90 41.9 -> 38.3,
+//    96 44.7 -> 38.2; 100 points 47.4 and 48.2.)
+//  * FP32 states over 24 MB take the TMA sweeps: their tiles stay in flight while
+//    others are solved, which pays once there are several per SM, in L2 (56 MB
+//    states are all hits) as from HBM (256^3 real 92 / 70 / 73 -> 59 / 48 / 49, 160
+//    x 144 x 150, 26 MB, imaginary 22.1 / 15.5 / 17.5 -> 17.5 / 11.3 / 14.9).  128^3
+//    (16 MB) is even at 29.4 us per step; 144 x 144 x 128 (20 MB) would gain
+//    already, 44.1 -> 36.9.
+//  * Smaller ones whose xy planes nearly fill the SMs take the fused x + y sweep
+//    (128^3 imaginary 13.2 + 7.7 -> 18.3).
 void choose_shapes_3d(gp_handle* h) {
   const int M0 = h->n[0] - 2, Ms = std::min(h->n[1], h->n[2]) - 2;
   if (h->prec == GP_F64) {

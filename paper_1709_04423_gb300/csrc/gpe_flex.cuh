@@ -7,9 +7,11 @@
 // power of two picked so that the tiles fill the SMs (flex_plan), times the
 // whole line, staged in shared memory; thread = (line, segment), any number of
 // segments per line that the block holds.  Per line the arithmetic is that of
-// tsweep_body / colsweep_body with the same segment length (bit for bit), with
-// more than 16 segments the carries' products are formed on the fly from the
-// segment products instead of read from the 16 x 16 tables.
+// tsweep_body / colsweep_body with the same segment length (bit for bit, but for
+// the sub-step N of FP64 states in imaginary time: from the whole angle here, in
+// factor form in tsweep_body, see phase_f64), with more than 16 segments the
+// carries' products are formed on the fly from the segment products instead of
+// read from the 16 x 16 tables.
 //
 // Tile layout: line c, point k at c P + k + (k - 1)/SEG (one element skipped
 // per segment; see flex_tile).  y/z tiles of W >= 2 (16-byte points) or 4

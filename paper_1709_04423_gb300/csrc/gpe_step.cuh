@@ -407,11 +407,12 @@ inline bool strang_close_fused(const gp_handle* h, bool imag) {
 //  * double-float 3d, lines over 130 points, in segments of 8 instead of 16 or 32:
 //    160 x 144 x 150 imaginary 122 / 58 / 67 -> 89 / 47 / 57, real 186 / 85 / 82 ->
 //    125 / 71 / 68 (its long dependent chains want more threads per line);
-//  * double-float x, fewer than 64 tiles: 257 x 201 37.8 -> 29.9; y would lose,
-//    19.0 -> 20.5.
+//  * double-float, fewer than 64 tiles: 257 x 201 imaginary time x 28.1 -> 9.0, y
+//    15.4 -> 7.2, real time 34.3 -> 15.2, 16.1 -> 13.1.
 // The plan picks the segments' length on 2d grids in imaginary time and on axial
-// ones; elsewhere they keep the handle's: Cartesian 2d real-time runs agree bit
-// for bit with the same run in a batch, and the shapes of a 3d grid with each other.
+// ones; elsewhere they keep the handle's, so that Cartesian 2d real-time runs agree
+// bit for bit with the same run in a batch, and the shapes of a 3d grid with each
+// other (but for double-float and, in imaginary time, FP64: see flex_body).
 template <typename T>
 FlexPlan flex_sweep(const gp_handle* h, bool imag, int d, int seg) {
   const int n = axis_len(h, d);
