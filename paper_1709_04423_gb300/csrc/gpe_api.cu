@@ -1548,6 +1548,8 @@ int gp_autotune(gp_handle* h, int imag, int nsteps, double* best_ms) {
     cudaError_t e = cudaMemcpyAsync(state, saved, sbytes, cudaMemcpyDeviceToDevice, h->work);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->work);
     if (e != cudaSuccess) rc = fail(GP_ERR_CUDA, cudaGetErrorString(e));
+    // a wait that gave up in a timed step: no shape was measured, the state is back
+    else rc = read_dev_err(h, "gp_autotune");
   }
   cudaFree(saved);
   const int best_flags = (best_k ? GP_SHAPE_KEEP_YZ : 0) | (best_px ? GP_SHAPE_PIPE_X : 0) |

@@ -103,3 +103,18 @@ def test_a_refused_tensor_map_is_an_error(G, phi0, monkeypatch, call):
     G.gp_test_refuse_maps(p.h, 0)
     recovers(G, p, phi0)
     p.close()
+
+
+def test_a_wait_that_ran_out_while_tuning_is_the_tuners_error(G, phi0, monkeypatch):
+    """The state is put back, so a read after it finds it and no error."""
+    p = default_handle(G, phi0, monkeypatch)
+    shapes = p.shapes()
+    G.gp_test_stall_transfers(p.h, 16)
+    with pytest.raises(G.GPError) as e:
+        G.gp_autotune(p.h, False, 1)
+    assert e.value.code == G.GP_ERR_TIMEOUT and "gp_autotune" in str(e.value)
+    G.gp_test_stall_transfers(p.h, 0)
+    assert p.shapes() == shapes
+    assert np.array_equal(p.get_state(device=False), phi0)
+    assert np.array_equal(p.get_state(device=True).cpu().numpy(), phi0)
+    p.close()
