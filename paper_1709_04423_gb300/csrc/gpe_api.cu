@@ -1257,9 +1257,10 @@ bool shapes_valid(const gp_handle* h, int tile_x, int seg_x, int seg_c) {
 }
 
 struct TuneKey {
-  int dim, n0, n1, n2, prec, imag, real;
+  int geom, dim, n0, n1, n2, prec, imag, real;
   bool operator<(const TuneKey& o) const {
-    return std::tie(dim, n0, n1, n2, prec, imag, real) < std::tie(o.dim, o.n0, o.n1, o.n2, o.prec, o.imag, o.real);
+    return std::tie(geom, dim, n0, n1, n2, prec, imag, real) <
+           std::tie(o.geom, o.dim, o.n0, o.n1, o.n2, o.prec, o.imag, o.real);
   }
 };
 std::map<TuneKey, std::array<int, 4>> g_tuned;  // process-wide results
@@ -1401,7 +1402,7 @@ int gp_autotune(gp_handle* h, int imag, int nsteps, double* best_ms) {
   if (nsteps < 1 || nsteps > 256) return fail(GP_ERR_INVALID, "gp_autotune: nsteps must be in [1, 256]");
   if (h->real_mode && !imag) return fail(GP_ERR_STATE, "gp_autotune: a real state takes imaginary-time steps only");
   const bool real = h->real_mode;  // tile x sweep, no pipelined shapes, the real buffer saved
-  const TuneKey key{h->dim, h->n[0], h->n[1], h->n[2], h->prec, imag != 0, real ? 1 : 0};
+  const TuneKey key{h->geom, h->dim, h->n[0], h->n[1], h->n[2], h->prec, imag != 0, real ? 1 : 0};
   {
     std::lock_guard<std::mutex> lock(g_tune_mutex);
     auto it = g_tuned.find(key);

@@ -441,6 +441,7 @@ class Propagator:
         if stream is None:
             stream = torch.cuda.current_stream()
         self.stream = stream
+        self.geometry = "spherical" if spherical else "axisym" if axisym else ""
         if spherical:
             if self.dim != 1:
                 raise ValueError("the spherical trap is a 1d radial problem")
@@ -546,7 +547,7 @@ class Propagator:
         path = os.environ.get("GPE_TUNE_CACHE", os.path.join(os.path.expanduser("~"), ".cache", "gpe_gb300",
                                                              "shapes.json"))
         # (the leading "narrow": entries made before the tiles of few lines were a shape lack their flags)
-        key = "|".join(["narrow", torch.cuda.get_device_name(), "x".join(map(str, self.n)), self.precision,
+        key = "|".join(["narrow", torch.cuda.get_device_name(), self.geometry + "x".join(map(str, self.n)), self.precision,
                         "imag" if imag else "real"] + (["real_state"] if self.real_state else []))
         table = {}
         if cache and os.path.exists(path):

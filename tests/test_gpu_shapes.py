@@ -109,6 +109,28 @@ def test_a_real_state_keeps_the_complex_shapes():
     p.close()
 
 
+def test_each_geometry_is_tuned_for_itself(tmp_path, monkeypatch):
+    """A Cartesian grid's tuned shapes (here the pipelined x sweep) are not those of an axial trap of the same size."""
+    from paper_1709_04423_gb300 import gpe as G
+    monkeypatch.setenv("GPE_TUNE_CACHE", str(tmp_path / "shapes.json"))
+    n, kw = [96, 4096 // 8], {"precision": "f64"}
+    c = G.Propagator(2, n, [0.1, 0.1], 1e-4, [1.0, 1.0], 5.0, **kw)
+    c.set_state(I.gaussian_state(2, n, [0.1, 0.1], [1.0, 1.0]))
+    c.autotune(True, nsteps=2)
+    import json
+    table = json.load(open(tmp_path / "shapes.json"))
+    key, = table
+    table[key] = dict(tile_x=1, seg_x=8, seg_c=32, flags=G.GP_SHAPE_PIPE_X)   # as the tuner may pick it
+    json.dump(table, open(tmp_path / "shapes.json", "w"))
+    assert c.autotune(True)["flags"] & G.GP_SHAPE_PIPE_X
+    a = G.Propagator(2, n, [0.1, 0.1], 1e-4, [1.0, 1.0], 5.0, axisym=True, **kw)
+    a.set_state(np.ones((n[1], n[0]), dtype=complex))
+    assert not a.autotune(True, nsteps=2)["flags"] & G.GP_SHAPE_PIPE_X
+    assert len(json.load(open(tmp_path / "shapes.json"))) == 2
+    c.close()
+    a.close()
+
+
 # imaginary time from 97 points on: FP32 rows with a pending factor arrive by cp.async
 @pytest.mark.parametrize("imag", [True, False])
 @pytest.mark.parametrize("prec", ["f64", "f32", "df64"])
