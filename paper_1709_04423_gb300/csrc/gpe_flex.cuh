@@ -311,11 +311,10 @@ __device__ __forceinline__ void flex_body(const Sweep2Args<T>& A, const FlexTile
     if (s < F.nseg) cbv[slot(s)] = z[0];
   }
   __syncthreads();
-  // FP32 states on grids with lines over 514 points (A.norm64): a thread's squares
-  // as SquareSum does, FP64 from there on
+  // FP32 states on grids with lines over 514 points (A.norm64): the norm by SquareSum
   constexpr bool kNorm64 = LAST && !CLOSE && std::is_same<T, float>::value;
   T nval = T(0);
-  [[maybe_unused]] double nval64 = 0.0;
+  [[maybe_unused]] SquareSum sq = SquareSum::zero();
   if (solving) {
     V Zin = vzero;
     if (small) {
@@ -370,18 +369,22 @@ __device__ __forceinline__ void flex_body(const Sweep2Args<T>& A, const FlexTile
         if constexpr (kNorm64) z[j] = u;
       }
       if constexpr (kNorm64) {
-        if (A.norm64 && solver) {
-          SquareSum sum;
+        if (A.norm64) {
+          float m = 0.f;
+          if (solver)
 #pragma unroll
-          for (int j = 0; j < SEG; ++j) sum.peak(z[j].x, z[j].y);  // (zeros past the line's end)
-          sum.scale();
+            for (int j = 0; j < SEG; ++j) m = fmaxf(m, fmaxf(fabsf(z[j].x), fabsf(z[j].y)));  // (zeros past the line)
+          sq.scale(m);
+          if (solver) {
+            const float wl = A.w_a[ci] * A.w_b[cf2];
 #pragma unroll
-          for (int j = 0; j < SEG; ++j) {
-            const float w = j < jm ? A.w_axis[k0 + j] : 0.f;
-            sum.add(w, z[j].x);
-            sum.add(w, z[j].y);
+            for (int j = 0; j < SEG; ++j) {
+              const float w = j < jm ? A.w_axis[k0 + j] * wl : 0.f;
+              sq.square(w, z[j].x);
+              sq.square(w, z[j].y);
+            }
           }
-          nval64 = sum.total() * ((double)A.w_a[ci] * A.w_b[cf2]);
+          sq.warp_total();
         }
       }
       if (s == 0 && solver && GPE_CHECK(base + (long)(n - 1) * st < lim, 304)) {
@@ -402,9 +405,13 @@ __device__ __forceinline__ void flex_body(const Sweep2Args<T>& A, const FlexTile
   }
   if constexpr (kNorm64) {
     if (A.norm64) {
-      double v[1] = {nval64};
-      block_sum<1>(v, red_smem);
-      if (tid == 0) A.parts_out[blockIdx.x] = v[0];
+      __shared__ SquareSum s_sq[kFlexMaxThreads / 32];
+      if (lane == 0) s_sq[warp] = sq;
+      __syncthreads();
+      if (warp == 0) {
+        sq = SquareSum::gather(s_sq, nwarps);
+        if (lane == 0) A.parts_out[blockIdx.x] = sq.value();
+      }
       return;
     }
   }

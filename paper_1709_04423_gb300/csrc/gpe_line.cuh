@@ -67,6 +67,7 @@ __device__ __forceinline__ unsigned cluster_rank() {
 template <typename V>
 __device__ __forceinline__ void st_cluster(V* dst, unsigned rank, V v) {
   static_assert(sizeof(V) == 4 || sizeof(V) == 8 || sizeof(V) == 16, "4, 8 or 16 bytes");
+  static_assert(alignof(V) == sizeof(V), "one aligned vector store");
   unsigned a;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((unsigned)__cvta_generic_to_shared(dst)), "r"(rank));
   unsigned w[sizeof(V) / 4];
@@ -97,11 +98,11 @@ __device__ __forceinline__ df64 line_rsqrt(df64 s) {
 }
 
 // The type a line's norm is summed in: the state precision (as a block's sums
-// are in the other kernels), and FP64 from each thread's SquareSum on for FP32
-// lines of more than 514 points, the ones with several points per thread (as on
-// the long lines of 2d and 3d grids; see flex_body).
+// are in the other kernels), and SquareSum for FP32 lines of more than 514 points,
+// the ones with several points per thread (as on the long lines of 2d and 3d
+// grids; see flex_body).
 template <typename T, int S>
-using line_norm_t = typename std::conditional<std::is_same<T, float>::value && (S > 1), double, T>::type;
+using line_norm_t = typename std::conditional<std::is_same<T, float>::value && (S > 1), SquareSum, T>::type;
 
 // The pending factor 1/sqrt(wscale * total) from the warps' norm sums in
 // shared memory, by every warp for itself: in FP64 from FP64 sums, in
@@ -109,6 +110,13 @@ using line_norm_t = typename std::conditional<std::is_same<T, float>::value && (
 // would take longer than the rest of the step).
 template <typename T>
 using line_scale_t = typename std::conditional<std::is_same<T, double>::value, double, df64>::type;
+
+__device__ __forceinline__ float line_factor(const SquareSum* nrm, int nparts, df64 ws) {
+  const SquareSum t = SquareSum::gather(nrm, nparts);
+  float h, l;
+  dfl::df_two_sum(t.s, t.c, h, l);
+  return line_rsqrt(df64(h, l + t.d) * ws).hi * SquareSum::pow2(-t.e);
+}
 
 template <typename T>
 __device__ __forceinline__ T line_factor(const T* nrm, int nparts, line_scale_t<T> ws) {
@@ -257,7 +265,7 @@ __global__ void __launch_bounds__(kLineMaxThreads) line_steps_kernel(const __gri
   for (long t = 0; t < P.nsteps; ++t) {
     // ---- the pending renormalisation and N
     if (IMAG && t > 0) {
-      const T scl = (T)line_factor<NT>(s_nrm, W, ws);
+      const T scl = line_factor(s_nrm, W, ws);
 #pragma unroll
       for (int j = 0; j < S; ++j) {
         p[j].x = p[j].x * scl;
@@ -391,30 +399,32 @@ __global__ void __launch_bounds__(kLineMaxThreads) line_steps_kernel(const __gri
 #pragma unroll
         for (int j = 0; j < S; ++j) p[j] = phase(p[j], j);
       }
-      NT nval = NT(0);
+      NT nval;
       if constexpr (std::is_same<NT, T>::value) {
+        nval = T(0);
 #pragma unroll
         for (int j = 0; j < S; ++j) nval = nval + wk[j] * (p[j].x * p[j].x + p[j].y * p[j].y);
-      } else {
-        SquareSum sum;
 #pragma unroll
-        for (int j = 0; j < S; ++j) sum.peak(p[j].x, p[j].y);
-        sum.scale();
+        for (int o = 16; o > 0; o >>= 1) nval = nval + shfl_xor_t(nval, o);
+      } else {
+        nval = NT::zero();
+        float m = 0.f;
+#pragma unroll
+        for (int j = 0; j < S; ++j) m = fmaxf(m, fmaxf(fabsf(p[j].x), fabsf(p[j].y)));
+        nval.scale(m);
 #pragma unroll
         for (int j = 0; j < S; ++j) {
-          sum.add(wk[j], p[j].x);
-          sum.add(wk[j], p[j].y);
+          nval.square(wk[j], p[j].x);
+          nval.square(wk[j], p[j].y);
         }
-        nval = sum.total();
+        nval.warp_total();
       }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) nval = nval + shfl_xor_t(nval, o);
       if (C > 1 || lane == 0) publish(s_nrm, w, nval);
       sync();  // third exchange
     }
   }
   if (IMAG) {
-    const T scl = (T)line_factor<NT>(s_nrm, W, ws);
+    const T scl = line_factor(s_nrm, W, ws);
 #pragma unroll
     for (int j = 0; j < S; ++j) {
       p[j].x = p[j].x * scl;
@@ -441,8 +451,8 @@ __global__ void __launch_bounds__(kLineMaxThreads) line_steps_kernel(const __gri
 //  * FP32: one block's barriers are cheaper than a cluster's, so a second block
 //    only from 512 threads of 4 points on (513 points, imaginary time: 1.58 with
 //    one block, 2.02 with four; 1000 real: 1.17 against 1.50; 4001 imaginary,
-//    before its norm's FP64 part: 2.58 with four blocks of 256 threads, 3.22 with
-//    two of 512; 4.22 now);
+//    with FP32 norm sums: 2.58 with four blocks of 256 threads, 3.22 with
+//    two of 512);
 //  * FP64 is bound by its two FP64 lanes per SM and the latency of its chain,
 //    so about 64 points per block (256 points: 5.63 with one block, 3.92 with
 //    four; 1000: 4.63 with eight, 6.81 with four), and more than one point per

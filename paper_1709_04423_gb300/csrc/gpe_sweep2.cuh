@@ -651,38 +651,69 @@ __device__ __forceinline__ void finish_norm(T tval, double* parts_out) {
   }
 }
 
-// Weighted squares of up to 64 FP32 values of any size, summed to FP64 accuracy
+// Weighted squares of FP32 values of any size, summed to FP64 accuracy and range
 // on the FP32 pipes: the norm of FP32 states on lines of more than 514 points,
-// which the thread-per-line kernels (gpe_sweep.cuh) sum in FP64.  The values
-// are scaled by the power of two that brings the largest to [1, 2) (peak, then
-// scale), so no square leaves the FP32 range that matters to the sum.  The weights
-// are Simpson coefficients, 0, 1, 2 and 4, so every weighted square is exactly a
-// pair of floats, and the pairs are summed with two levels of two-sums whose
-// errors go to a third word -- Ogita, Rump and Oishi's SumK with K = 3 (SIAM J.
-// Sci. Comput. 26, 2005), error below (64 2^-24)^3 = 2^-54 of the sum, against
-// up to n 2^-53 for n points summed in FP64.  About 50 FP32 operations per point
-// where FP64 takes six on a pipe of 1/70 the rate (conversions included): a
-// step of 1000 x 1000 points takes 37.2 us with this, 47.5 with FP64 sums and
-// 35.2 with FP32 ones, of 2000 points 5.7, 7.1 and 2.5.
-struct SquareSum {
-  float s = 0.f, c = 0.f, d = 0.f, m = 0.f, f = 1.f;
-  __device__ __forceinline__ void peak(float x, float y) { m = fmaxf(m, fmaxf(fabsf(x), fabsf(y))); }
-  // 2^-e for the largest value in [2^e, 2^(e+1)) (the ends of the range held so that 2^-e and the squares fit)
-  __device__ __forceinline__ void scale() {
-    const int b = min(max((int)(__float_as_uint(m) >> 23), 1), 253);
-    f = __uint_as_float((unsigned)(254 - b) << 23);
+// which the thread-per-line kernels (gpe_sweep.cuh) sum in FP64.  A sum is
+// (s + c + d) 2^(2e): the values of a warp are scaled by 2^-e, e the exponent of the
+// largest, so that no square leaves the FP32 range that matters to the sum.  The
+// weights are Simpson coefficients, 0, 1, 2 and 4, and products of them, so every
+// weighted square is exactly a pair of floats, and pairs, lanes and warps are
+// added with two levels of two-sums whose errors go to the third word -- Ogita,
+// Rump and Oishi's SumK with K = 3 (SIAM J. Sci. Comput. 26, 2005), error about
+// (n 2^-24)^3 of the sum for n terms, against up to n 2^-53 in FP64.  An FP64 sum
+// would take about 26 operations of every warp on a pipe that takes one per 19
+// clocks and SM.  us per imaginary-time step with FP32 sums, these, and FP64 sums
+// after each thread's squares: 2000 points 2.5, 3.5, 5.7; 4001 2.7, 3.2, 4.2; 1000 x
+// 1000 35.2, 37.1, 37.2.
+struct alignas(16) SquareSum {  // (stored whole, also to another block's shared memory)
+  float s, c, d;
+  int e;
+  static __device__ __forceinline__ SquareSum zero() { return SquareSum{0.f, 0.f, 0.f, -126}; }
+  // 2^k, 0 below the normal range
+  static __device__ __forceinline__ float pow2(int k) { return k < -126 ? 0.f : __uint_as_float((unsigned)(127 + k) << 23); }
+  // the scale of the warp's values, m the largest modulus of this lane's (the ends
+  // of the range held so that 2^-e and the squares fit); a warp calls it together
+  __device__ __forceinline__ void scale(float m) {
+    const int b = (int)(__reduce_max_sync(0xffffffffu, __float_as_uint(m)) >> 23);
+    e = min(max(b, 1), 253) - 127;
   }
-  __device__ __forceinline__ void add(float w, float v) {
-    const float x = v * f, h = x * x, p = w * h, e = w * fmaf(x, x, -h);
+  __device__ __forceinline__ void add(float hi, float lo) {
     float e1, e2, e3;
-    dfl::df_two_sum(s, p, s, e1);
+    dfl::df_two_sum(s, hi, s, e1);
     dfl::df_two_sum(c, e1, c, e2);
-    dfl::df_two_sum(c, e, c, e3);
+    dfl::df_two_sum(c, lo, c, e3);
     d += e2 + e3;
   }
-  __device__ __forceinline__ double total() const {
-    const int e = 127 - (int)(__float_as_uint(f) >> 23);
-    return ((double)s + ((double)c + (double)d)) * __hiloint2double((1023 + 2 * e) << 20, 0);  // 2^(2e)
+  __device__ __forceinline__ void square(float w, float v) {
+    const float x = v * pow2(-e), h = x * x;
+    add(w * h, w * fmaf(x, x, -h));
+  }
+  // the sum over the warp's lanes, at the warp's scale, in every lane
+  __device__ __forceinline__ void warp_total() {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const float so = __shfl_xor_sync(0xffffffffu, s, o), co = __shfl_xor_sync(0xffffffffu, c, o),
+                  dn = __shfl_xor_sync(0xffffffffu, d, o);
+      add(so, co);
+      d += dn;
+    }
+  }
+  // sums n others, each at its own scale, with a warp; the total is in every lane
+  static __device__ __forceinline__ SquareSum gather(const SquareSum* v, int n) {
+    const int lane = threadIdx.x & 31;
+    SquareSum t = zero();
+    for (int i = lane; i < n; i += 32) t.e = max(t.e, v[i].e);
+    t.e = __reduce_max_sync(0xffffffffu, t.e);
+    for (int i = lane; i < n; i += 32) {
+      const float f = pow2(2 * (v[i].e - t.e));
+      t.add(v[i].s * f, v[i].c * f);
+      t.d += v[i].d * f;
+    }
+    t.warp_total();
+    return t;
+  }
+  __device__ __forceinline__ double value() const {
+    return ((double)s + ((double)c + (double)d)) * __hiloint2double((1023 + 2 * e) << 20, 0);
   }
 };
 
