@@ -1449,6 +1449,7 @@ int gp_autotune(gp_handle* h, int imag, int nsteps, double* best_ms) {
   };
   // tiles of few lines, before the others: each plan once (several segment lengths
   // can lead to the same; with a y or z sweep that does not take them, per KEEP)
+  const bool x_tiles = !xs.empty() && xs[0][0] == 1;
   if (!real) {
     std::vector<std::array<int, 3>> seen;
     auto is_new = [&](int d0, int d1) {
@@ -1506,15 +1507,16 @@ int gp_autotune(gp_handle* h, int imag, int nsteps, double* best_ms) {
   int best_t = keep_t, best_x = keep_x, best_c = keep_c, best_k = keep_k, best_px = keep_px, best_pc = keep_pc;
   int best_tc = keep_tc, best_tx = keep_tx, best_nx = keep_nx, best_nc = keep_nc;
   // the sweeps are timed apart, without the overlap they have in a step, so a close
-  // call (5 %) stays with the tiles of few lines, whose rule was measured in steps
-  auto beats = [](double t, bool narrow, double best, bool best_narrow) {
-    return t < (best_narrow && !narrow ? 0.95 : 1.0) * best;
+  // call (5 %) stays with the tiles of few lines where the rule, which was measured
+  // in steps, has them (not where only the x tile was left out)
+  auto beats = [](double t, bool narrow, double best, bool best_by_rule) {
+    return t < (best_by_rule && !narrow ? 0.95 : 1.0) * best;
   };
   for (const auto& c : xs) {
     if (rc) break;
     double ms[3];
     rc = time_shape(c[0], c[1], c[2], c[3], c[4], keep_c, keep_k, keep_pc, keep_tc, keep_nc, ms);
-    if (!rc && beats(ms[0], c[4], bx, best_nx && bx < 1e30)) { bx = ms[0]; best_t = c[0]; best_x = c[1]; best_px = c[2]; best_tx = c[3]; best_nx = c[4]; }
+    if (!rc && beats(ms[0], c[4], bx, best_nx && (best_t || !x_tiles) && bx < 1e30)) { bx = ms[0]; best_t = c[0]; best_x = c[1]; best_px = c[2]; best_tx = c[3]; best_nx = c[4]; }
   }
   for (const auto& c : cs) {
     if (rc) break;
