@@ -388,8 +388,8 @@ int gp_observables_noalloc(int dim, const int n[3], const double dx[3], const do
  * sweep whose grid has few 32-line tiles runs on tiles of 1 to 16 lines, and
  * so does the x sweep of any grid without the x tile; on 1d grids GP_SHAPE_NARROW_X
  * runs every step of a call in one launch.  The segment length is the handle's
- * on Cartesian grids in real time and in 3d, else free.  gp_set_shapes drops
- * the flags where no sweep of the grid takes them; the pipelined, fused and
+ * on Cartesian grids in real time and in 3d, else free.  gp_get_shapes reports
+ * the flags where a sweep of the grid follows them; the pipelined, fused and
  * TMA forms of a sweep come before them.
  * gp_autotune times every valid shape of the x sweep and of the y/z
  * sweeps on this handle's grid (2 warm-up + nsteps timed steps each, imaginary

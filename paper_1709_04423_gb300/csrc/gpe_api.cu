@@ -486,22 +486,23 @@ bool takes_line(const gp_handle* h) {
 // Whether gp_step_* of this 1d grid runs in one launch (gpe_line.cuh).
 bool line_run(const gp_handle* h) { return h->dim == 1 && (h->seg_x == 0 || h->narrow_x) && takes_line(h); }
 
-// Sets narrow_x and narrow_c where wanted and where a sweep of the grid takes
-// them, so that gp_get_shapes reports what runs (a real state's sweeps never
-// do; its complex state keeps its flags).
+// Sets narrow_x and narrow_c (a real state's sweeps do not take them: its complex
+// state keeps its flags).
 void set_narrow(gp_handle* h, bool x, bool c) {
   if (h->real_mode) return;
   h->narrow_x = x && h->seg_x > 0;
   h->narrow_c = c && h->dim > 1 && h->seg_c > 0;
-  if (h->dim == 1) {
-    h->narrow_x = h->narrow_x && takes_line(h);
-    return;
-  }
+}
+
+// The GP_SHAPE_NARROW_* flags that a sweep of the grid follows, in either time
+// direction.
+int narrow_flags(const gp_handle* h) {
   auto taken = [&](int d) {
-    return sweep_kind_any(h, true, d) == SWEEP_NARROW || sweep_kind_any(h, false, d) == SWEEP_NARROW;
+    return d < h->dim &&
+           (sweep_kind_any(h, true, d) == SWEEP_NARROW || sweep_kind_any(h, false, d) == SWEEP_NARROW);
   };
-  h->narrow_x = h->narrow_x && taken(0);
-  h->narrow_c = h->narrow_c && (taken(1) || (h->dim > 2 && taken(2)));
+  return (h->narrow_x && (h->dim == 1 ? takes_line(h) : taken(0)) ? GP_SHAPE_NARROW_X : 0) |
+         (h->narrow_c && (taken(1) || taken(2)) ? GP_SHAPE_NARROW_YZ : 0);
 }
 
 // Defaults of 3d Cartesian grids, where the autotuner's picks agree over many
@@ -576,11 +577,11 @@ void choose_shapes(gp_handle* h) {
   h->pipe_x = pipe && h->tile_x && h->geom != 2 && pipe_fits(h, h->n[0], true);  // (no rho-axis pipelined sweep)
   h->xyfuse = env_int("GPE_FUSE_XY", 0) != 0 && plane_fits(h, sx);
   h->pipe_c = pipe && h->dim > 1 && sc > 0 && pipe_fits(h, nmax, false);
-  bool forced = false;
-  for (const char* e : {"GPE_TILE_X", "GPE_SEG_X", "GPE_SEG_YZ", "GPE_KEEP", "GPE_PIPE", "GPE_FUSE_XY"})
-    forced = forced || std::getenv(e);
-  if (h->dim == 3 && h->geom == 0 && !forced) choose_shapes_3d(h);
-  set_narrow(h, !forced, !forced);
+  bool forced_x = false, forced_c = false;
+  for (const char* e : {"GPE_TILE_X", "GPE_SEG_X", "GPE_PIPE", "GPE_FUSE_XY"}) forced_x = forced_x || std::getenv(e);
+  for (const char* e : {"GPE_SEG_YZ", "GPE_KEEP", "GPE_PIPE"}) forced_c = forced_c || std::getenv(e);
+  if (h->dim == 3 && h->geom == 0 && !forced_x && !forced_c) choose_shapes_3d(h);
+  set_narrow(h, !forced_x, !forced_c);
 }
 
 }  // namespace
@@ -641,7 +642,10 @@ int run_steps_any(gp_handle* h, bool imag, long nsteps) {
   return h->prec == GP_F64 ? run_steps_f64(h, imag, nsteps) : run_steps_f32(h, imag, nsteps);
 }
 int time_steps_any(gp_handle* h, bool imag, long nsteps, double* ms) {
-  if (line_run(h)) return time_line(h, imag, nsteps, ms);
+  if (line_run(h)) {
+    const int rc = time_line(h, imag, nsteps, ms);
+    if (rc != GP_ERR_STATE) return rc;
+  }
   if (h->prec == GP_DF64) return time_steps_df(h, imag, nsteps, ms);
   return h->prec == GP_F64 ? time_steps_f64(h, imag, nsteps, ms) : time_steps_f32(h, imag, nsteps, ms);
 }
@@ -1131,8 +1135,9 @@ int gp_time_sweeps_graph(gp_handle* h, int imag, int reps, double* ms_per_launch
     if (e != cudaSuccess) rc = fail(GP_ERR_CUDA, cudaGetErrorString(e));
   }
   if (!rc) {
-    rc = line_run(h)          ? time_line(h, imag != 0, reps, ms_per_launch)
-         : h->prec == GP_DF64 ? time_graph_df(h, imag != 0, reps, ms_per_launch)
+    rc = line_run(h) ? time_line(h, imag != 0, reps, ms_per_launch) : GP_ERR_STATE;
+    if (rc == GP_ERR_STATE)
+      rc = h->prec == GP_DF64 ? time_graph_df(h, imag != 0, reps, ms_per_launch)
          : h->prec == GP_F64 ? time_graph_f64(h, imag != 0, reps, ms_per_launch)
                              : time_graph_f32(h, imag != 0, reps, ms_per_launch);
   }
@@ -1378,7 +1383,7 @@ int gp_get_shapes(const gp_handle* h, int* tile_x, int* seg_x, int* seg_c, int* 
     *flags = (h->keep_c ? GP_SHAPE_KEEP_YZ : 0) | (h->pipe_x ? GP_SHAPE_PIPE_X : 0) |
              (h->pipe_c ? GP_SHAPE_PIPE_YZ : 0) | (h->xyfuse ? GP_SHAPE_FUSE_XY : 0) |
              (h->tma_c ? GP_SHAPE_TMA_YZ : 0) | (h->tma_x ? GP_SHAPE_TMA_X : 0) |
-             (h->narrow_x ? GP_SHAPE_NARROW_X : 0) | (h->narrow_c ? GP_SHAPE_NARROW_YZ : 0);
+             narrow_flags(h);
   return GP_OK;
 }
 
